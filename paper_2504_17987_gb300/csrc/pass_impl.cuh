@@ -644,13 +644,41 @@ __device__ __forceinline__ void sum_row_groups(float (&acc)[ND], int lrg)
     }
 }
 
+// Unit u of the plane loop as (block, shift row): whole groups of eight shift
+// rows of a block first, then every block's remaining ones.  The pitch of B' is
+// 4 x odd floats, so the 128-bit loads of a quarter-warp whose lanes take eight
+// consecutive rows of one block meet no bank twice; in plain block-major order
+// most quarter-warps straddle two blocks and meet some bank twice (16 px tiles
+// at r = 4: 7 wavefronts per load instead of 4.7; 16 pairs of 1 MP, 233 -> 218 us).
+template <int ND>
+__device__ __forceinline__ void plane_unit(int u, int nblk, int &b, int &syi)
+{
+    constexpr int M8 = ND & ~7, REM = ND - M8;
+    if (M8 == 0 || u < nblk * M8) {
+        constexpr int M = M8 ? M8 : ND;
+        b = u / M;
+        syi = u - b * M;
+    } else {
+        u -= nblk * M8;
+        b = u / REM;
+        syi = M8 + u - b * REM;
+    }
+}
+
 // Compile-time radius: each thread owns one (block, sy, row group) and keeps
 // the 2R+1 accumulators of its sx row in registers; rows are streamed from
 // shared memory four columns at a time with aligned 128-bit loads.
+// GT > 0: compile-time block size.  The loop is bound by the shared-memory pipe
+// (9 to 17 FMAs per loaded float), so a row's columns are unrolled and the B'
+// quads two neighbouring column quads share stay in registers: G / 4 + NQ - 1
+// quads per row instead of G / 4 * NQ (r = 6, 48 px windows: 10 instead of 30;
+// two 8 MP pairs, 678 -> 506 us, shared-memory pipe 86 -> 54 % busy; 24 px
+// windows 669 -> 540 us).
+// GT = 0: any block size that is a multiple of 4.
 // b0: first block (strips compute only the new block row after their first
 // step); ring_wy >= 0: strip mode, block row by of window row ring_wy goes to
 // ring row (ring_wy + by) & 1.
-template <int R>
+template <int R, int GT>
 __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs, float *Ps,
                                   int b0 = 0, int ring_wy = -1)
 {
@@ -658,15 +686,15 @@ __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileG
     constexpr int MIS = ((-R) % 4 + 4) % 4;
     constexpr int NQ = (4 + 2 * R + MIS + 3) / 4;
     const PassPlan &P = a.plan;
-    const int G = g.G, RG = P.RGx, rows = G / RG, lrg = __ffs(RG) - 1;
-    const int units = (g.nb - b0) * ND;  // (block, sy)
+    const int G = GT > 0 ? GT : g.G, RG = P.RGx, rows = G / RG, lrg = __ffs(RG) - 1;
+    const int nblk = g.nb - b0, units = nblk * ND;  // (block, sy)
     const int lane = threadIdx.x & 31, gi = lane >> (5 - lrg), ul = lane & ((32 >> lrg) - 1);
     // warp-uniform trip count for the shuffles; lanes past the last unit
     // repeat it and store nothing
     for (int base = (threadIdx.x - lane) >> lrg; base < units; base += blockDim.x >> lrg) {
-        const int u = min(base + ul, units - 1);
-        const int b = b0 + u / ND;
-        const int syi = u - (b - b0) * ND;
+        int b, syi;
+        plane_unit<ND>(min(base + ul, units - 1), nblk, b, syi);
+        b += b0;
         const int byi = b / g.nbx, bxi = b - byi * g.nbx;
         const int c0 = bxi * G, r0 = byi * G + gi * rows;
         // Two accumulator sets of packed pairs, so that every pair of B' values
@@ -679,38 +707,56 @@ __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileG
         float se = 0.f, so = 0.f;
 #pragma unroll
         for (int q = 0; q < NPR; ++q) pe[q] = po[q] = 0ull;
-        for (int y = r0; y < r0 + rows; ++y) {
-            const float *arow = As + y * P.a_pitch;
-            const float *brow = Bs + (y + syi + 1) * P.b_pitch + P.padl - R - MIS;
-            for (int c = c0; c < c0 + G; c += 4) {
-                const float4 a4 = *reinterpret_cast<const float4 *>(arow + c);
-                uint64_t bp[NQ * 2];
-                float bv[NQ * 4];
+        // four columns: A values a4 against the NQ quads of B' from w on
+        auto columns = [&](const float4 &a4, const float4 *w) {
+            uint64_t bp[NQ * 2];
+            float bv[NQ * 4];
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const float4 t = *reinterpret_cast<const float4 *>(brow + c + 4 * q);
-                    bv[4 * q] = t.x;
-                    bv[4 * q + 1] = t.y;
-                    bv[4 * q + 2] = t.z;
-                    bv[4 * q + 3] = t.w;
-                    bp[2 * q] = pack_f2(t.x, t.y);
-                    bp[2 * q + 1] = pack_f2(t.z, t.w);
-                }
-                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+            for (int q = 0; q < NQ; ++q) {
+                bv[4 * q] = w[q].x;
+                bv[4 * q + 1] = w[q].y;
+                bv[4 * q + 2] = w[q].z;
+                bv[4 * q + 3] = w[q].w;
+                bp[2 * q] = pack_f2(w[q].x, w[q].y);
+                bp[2 * q + 1] = pack_f2(w[q].z, w[q].w);
+            }
+            const float av[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint64_t a2 = pack_f2(av[j], av[j]);
-                    if (((MIS + j) & 1) == 0) {
+            for (int j = 0; j < 4; ++j) {
+                const uint64_t a2 = pack_f2(av[j], av[j]);
+                if (((MIS + j) & 1) == 0) {
 #pragma unroll
-                        for (int q = 0; q < NPR; ++q) pe[q] = ffma2(a2, bp[(MIS + j) / 2 + q], pe[q]);
-                        se = fmaf(av[j], bv[MIS + j + ND - 1], se);
-                    } else {
-                        so = fmaf(av[j], bv[MIS + j], so);
+                    for (int q = 0; q < NPR; ++q) pe[q] = ffma2(a2, bp[(MIS + j) / 2 + q], pe[q]);
+                    se = fmaf(av[j], bv[MIS + j + ND - 1], se);
+                } else {
+                    so = fmaf(av[j], bv[MIS + j], so);
 #pragma unroll
-                        for (int q = 0; q < NPR; ++q) po[q] = ffma2(a2, bp[(MIS + j + 1) / 2 + q], po[q]);
-                    }
+                    for (int q = 0; q < NPR; ++q) po[q] = ffma2(a2, bp[(MIS + j + 1) / 2 + q], po[q]);
                 }
             }
+        };
+        const float *arow = As + r0 * P.a_pitch + c0;
+        const float *brow = Bs + (r0 + syi + 1) * P.b_pitch + P.padl - R - MIS + c0;
+        for (int y = 0; y < rows; ++y) {
+            if (GT > 0) {
+                float4 w[GT / 4 + NQ];
+#pragma unroll
+                for (int q = 0; q < NQ - 1; ++q) w[q] = *reinterpret_cast<const float4 *>(brow + 4 * q);
+#pragma unroll
+                for (int q = 0; q < GT / 4; ++q) {
+                    w[q + NQ - 1] = *reinterpret_cast<const float4 *>(brow + 4 * (q + NQ - 1));
+                    columns(*reinterpret_cast<const float4 *>(arow + 4 * q), w + q);
+                }
+            } else {
+                for (int c = 0; c < G; c += 4) {
+                    float4 w[NQ];
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) w[q] = *reinterpret_cast<const float4 *>(brow + c + 4 * q);
+                    columns(*reinterpret_cast<const float4 *>(arow + c), w);
+                }
+            }
+            arow += P.a_pitch;
+            brow += P.b_pitch;
         }
         float acc[ND];
 #pragma unroll
@@ -732,6 +778,21 @@ __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileG
 #pragma unroll
             for (int d = 0; d < ND; ++d) out[d] = acc[d];
         }
+    }
+}
+
+// The plane loop of a kernel that is not specialised to one block size: the
+// block sizes of the usual windows (16 to 64 px at 50 % overlap, 32 to 96 px at
+// 75 %) run the unrolled loop.
+template <int R>
+__device__ __forceinline__ void block_planes_fp32_any(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs, float *Ps)
+{
+    switch (g.G) {
+    case 8: block_planes_fp32<R, 8>(a, g, As, Bs, Ps); return;
+    case 12: block_planes_fp32<R, 12>(a, g, As, Bs, Ps); return;
+    case 16: block_planes_fp32<R, 16>(a, g, As, Bs, Ps); return;
+    case 24: block_planes_fp32<R, 24>(a, g, As, Bs, Ps); return;
+    default: block_planes_fp32<R, 0>(a, g, As, Bs, Ps); return;
     }
 }
 
@@ -1470,8 +1531,10 @@ __global__ void __launch_bounds__(PASS_THREADS,
 
     // 3: block planes (alias the dead C region)
     if (PREC == PREC_FP32) {
-        if (RC >= 0)
-            block_planes_fp32<(RC >= 0 ? RC : 0)>(a, g, As, Bs, Ps);
+        if (RC >= 0 && GC > 0)
+            block_planes_fp32<(RC >= 0 ? RC : 0), GC>(a, g, As, Bs, Ps);
+        else if (RC >= 0)
+            block_planes_fp32_any<(RC >= 0 ? RC : 0)>(a, g, As, Bs, Ps);
         else
             block_planes_fp32_generic(a, g, As, Bs, Ps);
     } else {
@@ -1583,7 +1646,7 @@ __global__ void __launch_bounds__(PASS_THREADS, GC == 32 ? 3 : 4) strip_kernel(c
         // row items take their plane items after them)
         box_rows(a, g, Cs, Vs);
         window_stats(a, g, bst, stats, wy);
-        block_planes_fp32<RC>(a, g, As, Bs, Ps, k == 0 ? 0 : g.nbx, wy);
+        block_planes_fp32<RC, GC>(a, g, As, Bs, Ps, k == 0 ? 0 : g.nbx, wy);
         __syncthreads();
         // 4: plane, argmax, FP32 stencil, Gaussian fit, outputs
         // the direct stencil and its barrier only when some window needs them
