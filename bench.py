@@ -1052,6 +1052,10 @@ def kernel_bytes(rec: dict, bpp: int, margin: int) -> int | None:
     if name.startswith("down/"):  # a frame in (the input format at level 1, float above), its half out
         src = bpp if name == "down/L1" else 4
         return n * (W * H * src + (W // 2) * (H // 2) * 4)
+    if name.startswith("frames/"):  # frames read once; frame A as float (step) and the levels made (radius) written
+        src = bpp if name == "frames/L0" else 4
+        levels = sum((W >> k) * (H >> k) * 4 for k in range(1, rec["radius"] + 1))
+        return n * ((2 if rec["radius"] else 1) * W * H * src + rec["step"] * W * H * 4 + 2 * levels)
     if name.startswith("deform"):  # frame in, warped float frame with margins out
         src = 4 if "/L" in name else bpp
         return n * (W * H * src + (W + 2 * margin) * (H + 2 * margin) * 4)

@@ -312,9 +312,11 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
 
     // A, B: the images the warp samples; afl: frame A of the margin layout
     // (read by the pass when the first frame is not warped)
+    // src, n_src: the fields its predictor is interpolated from (0: none)
     auto run_pass = [&](const StageDef &d, PtrRef A, PtrRef B, int fmt, long long pch, PtrRef afl,
-                        bool pred) -> rpiv_status {
+                        const FieldSrc *src, int n_src) -> rpiv_status {
         const size_t n1 = (size_t)d.nx * d.ny;
+        const bool pred = n_src > 0;
         for (int which = central ? 0 : 1; which < 2; ++which) {
             DeformArgs da;
             std::memset(&da, 0, sizeof(da));
@@ -325,6 +327,8 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
             da.H = d.H;
             da.pred_u = pred ? ws(d.off_pred) : ptr_direct(nullptr, 0);
             da.pred_v = pred ? ws(d.off_pred + 4 * n1) : ptr_direct(nullptr, 0);
+            da.n_src = n_src;
+            for (int i = 0; i < n_src; ++i) da.src[i] = src[i];
             da.w = d.w;
             da.s = d.s;
             da.nx = d.nx;
@@ -393,28 +397,20 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
         CK(launch_uod(u, n, st), "outlier test launch");
         return RPIV_OK;
     };
-    auto run_interp = [&](const StageDef &src, PtrRef su, PtrRef sv, const StageDef &dst, int lv_up,
-                          int zero_if_null) -> rpiv_status {
-        InterpArgs ia;
-        const size_t nd = (size_t)dst.nx * dst.ny;
-        ia.su = su;
-        ia.sv = sv;
-        ia.snx = src.nx;
-        ia.sny = src.ny;
-        ia.sw = src.w;
-        ia.ss = src.s;
-        ia.du = ws(dst.off_pred);
-        ia.dv = ws(dst.off_pred + 4 * nd);
-        ia.dnx = dst.nx;
-        ia.dny = dst.ny;
-        ia.dw = dst.w;
-        ia.ds = dst.s;
-        ia.levels_up = lv_up;
-        ia.zero_if_null = zero_if_null;
-        TraceScope ts(h, st, "interp/" + stage_tag(h, dst),
-                      geom_of(dst.W, dst.H, dst.w, dst.s, dst.R, dst.nx, dst.ny, n));
-        CK(launch_interp(ia, n, st), "interpolation launch");
-        return RPIV_OK;
+    // the validated field of a stage, or (fin) the caller's predictor on the final grid
+    auto field_of = [&](const StageDef &d, PtrRef u, PtrRef v, int lv_up) {
+        FieldSrc f;
+        f.u = u;
+        f.v = v;
+        f.nx = d.nx;
+        f.ny = d.ny;
+        f.w = d.w;
+        f.s = d.s;
+        f.levels_up = lv_up;
+        return f;
+    };
+    auto validated = [&](const StageDef &d, int lv_up) {
+        return field_of(d, ws(d.off_out), ws(d.off_out + 4 * (size_t)d.nx * d.ny), lv_up);
     };
     rpiv_status rs;
 
@@ -439,90 +435,69 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
         img_pitch = h->in_pitch;
     }
 
-    bool pass0_pred = false;
-    if (!central) {
-        // frame A as float, read by every full-resolution pass
-        IngestArgs ia;
-        ia.src = img_a;
-        ia.fmt = user_fmt;
-        ia.pitch = img_pitch;
-        ia.W = c.width;
-        ia.H = c.height;
-        ia.dst = ws(h->frame_off[0][0]);
-        ia.dst_pitch = p0.fpitch;
-        ia.dst_margin = M;
-        TraceScope ts(h, st, "ingest", geom_of(c.width, c.height, 0, 0, 0, 0, 0, n));
-        CK(launch_ingest(ia, n, st), "ingest launch");
-    }
-    if (run_pyr) {
-        for (int l = 1; l <= L; ++l) {
-            const StageDef &cur = h->stages[L - l];
-            for (int ab = 0; ab < 2; ++ab) {
-                DownArgs d;
-                if (l == 1) {
-                    d.src = ab ? img_b : img_a;
-                    d.fmt = user_fmt;
-                    d.pitch = img_pitch;
-                    d.W = c.width;
-                    d.H = c.height;
-                } else {
-                    const StageDef &prev = h->stages[L - (l - 1)];
-                    d.src = ws(h->frame_off[l - 1][ab] + interior(prev.fpitch));
-                    d.fmt = PIX_F32;
-                    d.pitch = prev.fpitch * 4;
-                    d.W = prev.W;
-                    d.H = prev.H;
-                }
-                d.dst = ws(h->frame_off[l][ab]);
-                d.dst_pitch = cur.fpitch;
-                d.dst_margin = M;
-                TraceScope ts(h, st, "down/L" + std::to_string(l), geom_of(d.W, d.H, 0, 0, 0, 0, 0, n));
-                CK(launch_down(d, n, st), "pyramid launch");
-            }
+    // frame A as float, read by every full-resolution pass, and the pyramid: two
+    // levels per launch, the first with frame A
+    for (int l = 0; l == 0 || (run_pyr && l < L); l += 2) {
+        FramesArgs fa;
+        std::memset(&fa, 0, sizeof(fa));
+        fa.margin = M;
+        fa.levels = run_pyr ? std::min(2, L - l) : 0;
+        fa.frames = fa.levels > 0 ? 2 : 1;
+        if (l == 0) {
+            if (central && !run_pyr) break;
+            fa.src[0] = img_a;
+            fa.src[1] = img_b;
+            fa.fmt = user_fmt;
+            fa.pitch = img_pitch;
+            fa.W = c.width;
+            fa.H = c.height;
+            fa.ingest = central ? 0 : 1;
+            fa.full = ws(h->frame_off[0][0]);
+            fa.full_pitch = p0.fpitch;
+        } else {
+            const StageDef &prev = h->stages[L - l];
+            for (int ab = 0; ab < 2; ++ab) fa.src[ab] = ws(h->frame_off[l][ab] + interior(prev.fpitch));
+            fa.fmt = PIX_F32;
+            fa.pitch = prev.fpitch * 4;
+            fa.W = prev.W;
+            fa.H = prev.H;
         }
+        for (int k = 0; k < fa.levels; ++k) {
+            for (int ab = 0; ab < 2; ++ab) fa.down[k][ab] = ws(h->frame_off[l + k + 1][ab]);
+            fa.down_pitch[k] = h->stages[L - (l + k + 1)].fpitch;
+        }
+        // the record's radius and step: levels made, frame A made
+        TraceScope ts(h, st, "frames/L" + std::to_string(l), geom_of(fa.W, fa.H, 0, fa.ingest, fa.levels, 0, 0, n));
+        CK(launch_frames(fa, n, st), "frames launch");
+    }
+    FieldSrc src[2];
+    int n_src = 0;
+    if (run_pyr) {
         for (int i = 0; i < L; ++i) {
             const StageDef &d = h->stages[i];
-            const bool pred = i > 0;
-            if (pred) {
-                const StageDef &prev = h->stages[i - 1];
-                const size_t np = (size_t)prev.nx * prev.ny;
-                if ((rs = run_interp(prev, ws(prev.off_out), ws(prev.off_out + 4 * np), d, 1, 0)) != RPIV_OK) return rs;
-            }
+            if (i > 0) src[n_src++] = validated(h->stages[i - 1], 1);
             const size_t in = interior(d.fpitch);
             if ((rs = run_pass(d, ws(h->frame_off[d.lvl][0] + in), ws(h->frame_off[d.lvl][1] + in), PIX_F32,
-                               d.fpitch * 4, ws(h->frame_off[d.lvl][0]), pred)) != RPIV_OK)
+                               d.fpitch * 4, ws(h->frame_off[d.lvl][0]), src, n_src)) != RPIV_OK)
                 return rs;
             if ((rs = run_uod(d, false)) != RPIV_OK) return rs;
+            n_src = 0;
         }
-        const StageDef &l1 = h->stages[L - 1];
-        const size_t n1 = (size_t)l1.nx * l1.ny;
-        if ((rs = run_interp(l1, ws(l1.off_out), ws(l1.off_out + 4 * n1), p0, 1, 0)) != RPIV_OK) return rs;
-        pass0_pred = true;
+        src[n_src++] = validated(h->stages[L - 1], 1);
     }
-    if (any_pred) {
-        // caller predictor on the final-pass grid; pairs without one keep the
-        // pyramid result, or get zero when there is no pyramid
-        const StageDef &fin = h->stages.back();
-        if ((rs = run_interp(fin, tab(&io[0].pred_u), tab(&io[0].pred_v), p0, 0, run_pyr ? 0 : 1)) != RPIV_OK)
-            return rs;
-        pass0_pred = true;
-    }
+    // caller predictor on the final-pass grid; pairs without one take the
+    // pyramid result, or zero when there is no pyramid
+    if (any_pred) src[n_src++] = field_of(h->stages.back(), tab(&io[0].pred_u), tab(&io[0].pred_v), 0);
     const int np = c.n_passes;
     for (int p = 0; p < np; ++p) {
         const StageDef &d = h->stages[L + p];
-        bool pred = (p == 0) ? pass0_pred : true;
         if (p > 0) {
-            const StageDef &prev = h->stages[L + p - 1];
-            const size_t nprev = (size_t)prev.nx * prev.ny;
-            if ((rs = run_interp(prev, ws(prev.off_out), ws(prev.off_out + 4 * nprev), d, 0, 0)) != RPIV_OK) return rs;
+            src[0] = validated(h->stages[L + p - 1], 0);
+            n_src = 1;
         }
-        if ((rs = run_pass(d, img_a, img_b, user_fmt, img_pitch, ws(h->frame_off[0][0]),
-                           pred)) != RPIV_OK)
+        if ((rs = run_pass(d, img_a, img_b, user_fmt, img_pitch, ws(h->frame_off[0][0]), src, n_src)) != RPIV_OK)
             return rs;
         if ((rs = run_uod(d, p == np - 1)) != RPIV_OK) return rs;
-        if (p < np - 1) {
-            // the next pass reads this pass's validated field from the workspace
-        }
     }
     const StageDef &fin = h->stages.back();
     VortArgs va;
@@ -614,16 +589,19 @@ int rpiv::single_pass(const void *img_a, const void *img_b, size_t pitch_bytes, 
     const int pfmt = fmt == RPIV_U8 ? PIX_U8 : (fmt == RPIV_U16 ? PIX_U16 : PIX_F32);
     prepare_pass_kernels();
     if (!central) {
-        IngestArgs ia;
-        ia.src = ptr_direct(img_a, 0);
-        ia.fmt = pfmt;
-        ia.pitch = (long long)pitch_bytes;
-        ia.W = width;
-        ia.H = height;
-        ia.dst = ptr_direct(first, 0);
-        ia.dst_pitch = fp;
-        ia.dst_margin = M;
-        CK(launch_ingest(ia, 1, st), "ingest launch");
+        FramesArgs fa;
+        std::memset(&fa, 0, sizeof(fa));
+        fa.src[0] = ptr_direct(img_a, 0);
+        fa.frames = 1;
+        fa.fmt = pfmt;
+        fa.pitch = (long long)pitch_bytes;
+        fa.W = width;
+        fa.H = height;
+        fa.margin = M;
+        fa.ingest = 1;
+        fa.full = ptr_direct(first, 0);
+        fa.full_pitch = fp;
+        CK(launch_frames(fa, 1, st), "ingest launch");
     }
     for (int which = central ? 0 : 1; which < 2; ++which) {
         DeformArgs da;
@@ -1375,16 +1353,18 @@ rpiv_status rpiv_stage_downsample(const void *img, size_t pitch_bytes, int fmt, 
     if (fmt != 0 && fmt != RPIV_U8 && fmt != RPIV_U16) return fail(RPIV_ERR_INVALID_ARG, "fmt");
     const int bpp = fmt == RPIV_U8 ? 1 : (fmt == RPIV_U16 ? 2 : 4);
     if (pitch_bytes < (size_t)width * bpp) return fail(RPIV_ERR_INVALID_ARG, "pitch_bytes");
-    DownArgs a;
-    a.src = ptr_direct(img, 0);
+    FramesArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.src[0] = ptr_direct(img, 0);
+    a.frames = 1;
     a.fmt = fmt == RPIV_U8 ? PIX_U8 : (fmt == RPIV_U16 ? PIX_U16 : PIX_F32);
     a.pitch = (long long)pitch_bytes;
     a.W = width;
     a.H = height;
-    a.dst = ptr_direct(out, 0);
-    a.dst_pitch = width / 2;
-    a.dst_margin = 0;
-    CK(launch_down(a, 1, static_cast<cudaStream_t>(cuda_stream)), "downsample launch");
+    a.levels = 1;
+    a.down[0][0] = ptr_direct(out, 0);
+    a.down_pitch[0] = width / 2;
+    CK(launch_frames(a, 1, static_cast<cudaStream_t>(cuda_stream)), "downsample launch");
     return RPIV_OK;
 }
 

@@ -14,6 +14,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "grid_interp.cuh"
 #include "rpiv_internal.h"
 
 namespace rpiv {
@@ -34,16 +35,14 @@ constexpr int nrow_cap(int dty, int min_step) { return dty / min_step + 4; }
 
 // cell index and weight of a pixel position along one axis of the node grid
 // (node i at c0 + i s; positions outside the hull take the border value)
-// (the division stays: a rounded reciprocal of a step that is not a power of
-// two would bias every weight the same way, up to 1e-5 px at 4k columns)
-__device__ __forceinline__ void axis_weight(int pos, int n, float c0, float s, int &i0, float &t)
+__device__ __forceinline__ void axis_weight(int pos, int n, float c0, int s, int &i0, float &t)
 {
     if (n <= 1) {
         i0 = 0;
         t = 0.f;
         return;
     }
-    float f = ((float)pos - c0) / s;
+    float f = over_step((float)pos - c0, s);
     f = fminf(fmaxf(f, 0.f), (float)(n - 1));
     int ia = (int)floorf(f);
     if (ia > n - 2) ia = n - 2;
@@ -207,12 +206,14 @@ __device__ __forceinline__ void deform_rows_any(const DeformArgs &a, const T *ba
 // The field is bilinear in the nodes: the tile first interpolates every node
 // row it touches along x at each of its columns, already scaled (cuv), and
 // stores per row its node-row offset and weight (rinfo), so that a pixel needs
-// one interpolation along y.  A tile whose taps provably stay inside the image
+// one interpolation along y.  With a source field (n_src) the tile interpolates
+// its nodes from it, and stores them for the pass (as a launch of its own the
+// interpolation of a single pair took as long as a small pass).  A tile whose taps provably stay inside the image
 // (its displacement lies within the range of its nodes, a convex combination)
 // skips the clamping; either way every tap is the clamp-to-edge sample.
 template <typename T, int DTY, int MIN_STEP>
-__device__ void deform_tile(const DeformArgs &a, const unsigned char *img, const float *pu, const float *pv,
-                            float *out)
+__device__ void deform_tile(const DeformArgs &a, const unsigned char *img, float *pu, float *pv, float *out,
+                            int pair)
 {
     constexpr int NCAP = MIN_STEP >= 8 ? NODE_CAP_S8 : NODE_CAP;
     __shared__ float nu[NCAP], nv[NCAP];
@@ -220,7 +221,7 @@ __device__ void deform_tile(const DeformArgs &a, const unsigned char *img, const
     __shared__ __align__(16) int2 rinfo[DTY];
     __shared__ float red[4][8];
     const int x0 = blockIdx.x * DTX - a.M, y0 = blockIdx.y * DTY - a.M;
-    const float c0 = 0.5f * (float)(a.w - 1), sf = (float)a.s;
+    const float c0 = 0.5f * (float)(a.w - 1);
     const bool has = pu != nullptr && pv != nullptr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lx = threadIdx.x % DTX, ly0 = threadIdx.x / DTX;
@@ -231,18 +232,36 @@ __device__ void deform_tile(const DeformArgs &a, const unsigned char *img, const
     if (has) {
         int ilo, ihi, jlo, jhi;
         float t;
-        axis_weight(x0, a.nx, c0, sf, ilo, t);
-        axis_weight(x0 + DTX - 1, a.nx, c0, sf, ihi, t);
-        axis_weight(y0, a.ny, c0, sf, jlo, t);
-        axis_weight(y0 + DTY - 1, a.ny, c0, sf, jhi, t);
+        axis_weight(x0, a.nx, c0, a.s, ilo, t);
+        axis_weight(x0 + DTX - 1, a.nx, c0, a.s, ihi, t);
+        axis_weight(y0, a.ny, c0, a.s, jlo, t);
+        axis_weight(y0 + DTY - 1, a.ny, c0, a.s, jhi, t);
         ihi = min(ihi + 1, a.nx - 1);
         jhi = min(jhi + 1, a.ny - 1);
         const int nwn = ihi - ilo + 1, nhn = jhi - jlo + 1;
         float lu0 = INFINITY, lu1 = -INFINITY, lv0 = INFINITY, lv1 = -INFINITY;
         bool nan_seen = false;
+        const FieldSrc &fs = a.src[a.n_src > 1 && resolve(a.src[1].u, pair) && resolve(a.src[1].v, pair) ? 1 : 0];
+        const float *su = nullptr, *sv = nullptr;
+        if (a.n_src > 0) {
+            su = (const float *)resolve(fs.u, pair);
+            sv = (const float *)resolve(fs.v, pair);
+            if (!sv) su = nullptr;
+        }
         for (int e = threadIdx.x; e < nwn * nhn; e += blockDim.x) {
             const int jj = e / nwn, ii = e - jj * nwn;
-            const float fu = pu[(jlo + jj) * a.nx + ilo + ii], fv = pv[(jlo + jj) * a.nx + ilo + ii];
+            const int node = (jlo + jj) * a.nx + ilo + ii;
+            float fu, fv;
+            if (a.n_src > 0) {
+                // the tiles that share a node write the same value
+                const float2 d = su ? interp_node(su, sv, fs.nx, fs.ny, fs.w, fs.s, a.w, a.s, fs.levels_up, ilo + ii, jlo + jj)
+                                    : make_float2(0.f, 0.f);
+                pu[node] = fu = d.x;
+                pv[node] = fv = d.y;
+            } else {
+                fu = pu[node];
+                fv = pv[node];
+            }
             nu[e] = fu;
             nv[e] = fv;
             nan_seen |= (fu != fu) || (fv != fv);
@@ -263,7 +282,7 @@ __device__ void deform_tile(const DeformArgs &a, const unsigned char *img, const
         }
         for (int e = threadIdx.x; e < DTY; e += blockDim.x) {
             int j0;
-            axis_weight(y0 + e, a.ny, c0, sf, j0, t);
+            axis_weight(y0 + e, a.ny, c0, a.s, j0, t);
             rinfo[e] = make_int2((j0 - jlo) * DTX, __float_as_int(t));
         }
         any_nan = __syncthreads_or(nan_seen);
@@ -271,7 +290,7 @@ __device__ void deform_tile(const DeformArgs &a, const unsigned char *img, const
         {
             int i0;
             float tx;
-            axis_weight(x, a.nx, c0, sf, i0, tx);
+            axis_weight(x, a.nx, c0, a.s, i0, tx);
             const int ci = i0 - ilo, di = a.nx > 1 ? 1 : 0;
             for (int jj = ly0; jj < nhn; jj += blockDim.x / DTX) {
                 const float *ru = nu + jj * nwn + ci, *rv = nv + jj * nwn + ci;
@@ -326,10 +345,10 @@ __global__ void __launch_bounds__(256, 6) deform_kernel(const DeformArgs a)
 {
     const int pair = blockIdx.z;
     const unsigned char *img = (const unsigned char *)resolve(a.img, pair);
-    const float *pu = (const float *)resolve(a.pred_u, pair);
-    const float *pv = (const float *)resolve(a.pred_v, pair);
+    float *pu = (float *)resolve(a.pred_u, pair);
+    float *pv = (float *)resolve(a.pred_v, pair);
     float *out = (float *)resolve(a.out, pair);
-    deform_tile<T, DTY, MIN_STEP>(a, img, pu, pv, out);
+    deform_tile<T, DTY, MIN_STEP>(a, img, pu, pv, out, pair);
 }
 
 // nodes touched by a DTX x dty tile along each axis, plus the neighbour node,

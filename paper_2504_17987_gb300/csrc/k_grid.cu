@@ -9,6 +9,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "grid_interp.cuh"
 #include "rpiv_internal.h"
 
 namespace rpiv {
@@ -167,22 +168,6 @@ cudaError_t launch_uod(const UodArgs &a, int n_pairs, cudaStream_t st)
 
 // --------------------------------------------------------------- interp --
 
-__device__ __forceinline__ void axis_wf(float pos, int n, float c0, int s, int &i0, int &i1, float &t)
-{
-    if (n <= 1) {
-        i0 = i1 = 0;
-        t = 0.f;
-        return;
-    }
-    float f = (pos - c0) / (float)s;
-    f = fminf(fmaxf(f, 0.f), (float)(n - 1));
-    int ia = (int)floorf(f);
-    if (ia > n - 2) ia = n - 2;
-    i0 = ia;
-    i1 = ia + 1;
-    t = f - (float)ia;
-}
-
 __global__ void interp_kernel(const InterpArgs a)
 {
     const int pair = blockIdx.y;
@@ -200,21 +185,9 @@ __global__ void interp_kernel(const InterpArgs a)
         return;
     }
     const int j = k / a.dnx, i = k - j * a.dnx;
-    const float f = (float)(1 << a.levels_up);
-    const float X = (float)(i * a.ds) + 0.5f * (float)(a.dw - 1);
-    const float Y = (float)(j * a.ds) + 0.5f * (float)(a.dw - 1);
-    const float xs = (X + 0.5f) / f - 0.5f, ys = (Y + 0.5f) / f - 0.5f;
-    const float c0 = 0.5f * (float)(a.sw - 1);
-    int i0, i1, j0, j1;
-    float tx, ty;
-    axis_wf(xs, a.snx, c0, a.ss, i0, i1, tx);
-    axis_wf(ys, a.sny, c0, a.ss, j0, j1, ty);
-    float t0 = su[j0 * a.snx + i0] + tx * (su[j0 * a.snx + i1] - su[j0 * a.snx + i0]);
-    float t1 = su[j1 * a.snx + i0] + tx * (su[j1 * a.snx + i1] - su[j1 * a.snx + i0]);
-    du[k] = f * (t0 + ty * (t1 - t0));
-    t0 = sv[j0 * a.snx + i0] + tx * (sv[j0 * a.snx + i1] - sv[j0 * a.snx + i0]);
-    t1 = sv[j1 * a.snx + i0] + tx * (sv[j1 * a.snx + i1] - sv[j1 * a.snx + i0]);
-    dv[k] = f * (t0 + ty * (t1 - t0));
+    const float2 d = interp_node(su, sv, a.snx, a.sny, a.sw, a.ss, a.dw, a.ds, a.levels_up, i, j);
+    du[k] = d.x;
+    dv[k] = d.y;
 }
 
 cudaError_t launch_interp(const InterpArgs &a, int n_pairs, cudaStream_t st)
@@ -277,122 +250,109 @@ cudaError_t launch_vort(const VortArgs &a, int n_pairs, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------- downsample --
+// --------------------------------------------- frames and their pyramid --
 
+// Four consecutive source pixels of a row from pixel p (a multiple of 4): one
+// 4-byte (u8), 8-byte (u16) or 16-byte (float) load.
 template <typename T>
-__device__ __forceinline__ float ldp(const unsigned char *img, long long pitch, int x, int y)
-{
-    return (float)__ldg(reinterpret_cast<const T *>(img + (long long)y * pitch) + x);
-}
-
-template <typename T>
-__device__ __forceinline__ float box2(const unsigned char *img, long long pitch, int x, int y)
-{
-    // (a + b + c + d) / 4 is exact in FP32 for integer (or quarter-integer) pixels
-    return 0.25f * ((ldp<T>(img, pitch, 2 * x, 2 * y) + ldp<T>(img, pitch, 2 * x + 1, 2 * y)) +
-                    (ldp<T>(img, pitch, 2 * x, 2 * y + 1) + ldp<T>(img, pitch, 2 * x + 1, 2 * y + 1)));
-}
-
-// Eight consecutive source pixels of a row from pixel p (p a multiple of 8):
-// one 8-byte (u8), 16-byte (u16) or two 16-byte (float) loads.
-template <typename T>
-__device__ __forceinline__ void load8(const unsigned char *row, int p, float (&v)[8])
+__device__ __forceinline__ void load4(const unsigned char *row, int p, float (&v)[4])
 {
     if (sizeof(T) == 1) {
-        const uint2 u = __ldg(reinterpret_cast<const uint2 *>(row) + p / 8);
+        const uint32_t u = __ldg(reinterpret_cast<const uint32_t *>(row) + p / 4);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[i] = (float)((u.x >> (8 * i)) & 0xffu);
-            v[4 + i] = (float)((u.y >> (8 * i)) & 0xffu);
-        }
+        for (int i = 0; i < 4; ++i) v[i] = (float)((u >> (8 * i)) & 0xffu);
     } else if (sizeof(T) == 2) {
-        const uint4 u = __ldg(reinterpret_cast<const uint4 *>(row) + p / 8);
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[2 * i] = (float)(w[i] & 0xffffu);
-            v[2 * i + 1] = (float)(w[i] >> 16);
-        }
+        const uint2 u = __ldg(reinterpret_cast<const uint2 *>(row) + p / 4);
+        v[0] = (float)(u.x & 0xffffu);
+        v[1] = (float)(u.x >> 16);
+        v[2] = (float)(u.y & 0xffffu);
+        v[3] = (float)(u.y >> 16);
     } else {
-        const float4 f0 = __ldg(reinterpret_cast<const float4 *>(row) + p / 4);
-        const float4 f1 = __ldg(reinterpret_cast<const float4 *>(row) + p / 4 + 1);
-        v[0] = f0.x; v[1] = f0.y; v[2] = f0.z; v[3] = f0.w;
-        v[4] = f1.x; v[5] = f1.y; v[6] = f1.z; v[7] = f1.w;
+        const float4 f = __ldg(reinterpret_cast<const float4 *>(row) + p / 4);
+        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
     }
 }
 
-// Four consecutive outputs per thread (x0 = 4 k): their 2 x 8 source pixels by
-// one vector load per source row and one 16-byte store, where the source rows
-// and the destination row are aligned for them (checked per pair); the row's
-// last outputs and unaligned rows take the scalar form.  Same sums, in the
-// same order, either way.
-template <typename T>
-__device__ __forceinline__ void down_row4(const unsigned char *src, long long pitch, int x0, int y, int W2, float *d,
-                                          bool vec)
+// The first n of N consecutive floats to d: one vector store where d is aligned
+// for it and all are wanted.
+template <int N>
+__device__ __forceinline__ void store_run(float *d, const float (&v)[N], int n)
 {
-    if (vec && x0 + 4 <= W2) {
-        float r0[8], r1[8];
-        load8<T>(src + (long long)(2 * y) * pitch, 2 * x0, r0);
-        load8<T>(src + (long long)(2 * y + 1) * pitch, 2 * x0, r1);
-        float o[4];
+    if (N == 4 && n >= N && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+        *reinterpret_cast<float4 *>(d) = make_float4(v[0], v[1], v[N - 2], v[N - 1]);
+    } else if (N == 2 && n >= N && (reinterpret_cast<uintptr_t>(d) & 7) == 0) {
+        *reinterpret_cast<float2 *>(d) = make_float2(v[0], v[N - 1]);
+    } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) o[i] = 0.25f * ((r0[2 * i] + r0[2 * i + 1]) + (r1[2 * i] + r1[2 * i + 1]));
-        *reinterpret_cast<float4 *>(d) = make_float4(o[0], o[1], o[2], o[3]);
-        return;
+        for (int i = 0; i < N; ++i)
+            if (i < n) d[i] = v[i];
     }
-    for (int k = 0; k < 4 && x0 + k < W2; ++k) d[k] = box2<T>(src, pitch, x0 + k, y);
 }
 
-__global__ void __launch_bounds__(256) down_kernel(const DownArgs a)
-{
-    const int pair = blockIdx.z;
-    const int W2 = a.W / 2, H2 = a.H / 2;
-    const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x0 >= W2 || y >= H2) return;
-    const unsigned char *src = (const unsigned char *)resolve(a.src, pair);
-    float *dst = (float *)resolve(a.dst, pair);
-    float *d = dst + (long long)(y + a.dst_margin) * a.dst_pitch + (x0 + a.dst_margin);
-    const int bpp = a.fmt == PIX_U8 ? 1 : (a.fmt == PIX_U16 ? 2 : 4);
-    const int align = bpp == 1 ? 8 : 16;
-    const bool vec = ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)a.pitch) % align) == 0 &&
-                     (reinterpret_cast<uintptr_t>(d) % 16) == 0;
-    if (a.fmt == PIX_U8) down_row4<uint8_t>(src, a.pitch, x0, y, W2, d, vec);
-    else if (a.fmt == PIX_U16) down_row4<uint16_t>(src, a.pitch, x0, y, W2, d, vec);
-    else down_row4<float>(src, a.pitch, x0, y, W2, d, vec);
-}
+// A thread takes a patch of 4 x 4 source pixels (one vector load per row where
+// the rows are aligned for it): frame A's floats, 2 x 2 pixels of level 1 and
+// one of level 2, so that a frame is read once for all three and a warp's
+// stores are contiguous.  Each level is the 2x2 box mean of the one below,
+// ((a + b) + (c + d)) / 4.  Bound by DRAM: 64 pairs of 1 MP u16, two levels,
+// 705 MB in 117 us (0.88 of the measured copy rate); patches of 8 x 4 took 157
+// us (half-filled sectors per store), of 4 x 8 134 us (fewer warps).  As five
+// launches (frame A, levels 1 and 2 of each frame) it was 195 us, and five of
+// the 23 launches of a single pair.
+constexpr int FR_ROWS = 4;
 
-// Eight consecutive pixels per thread: one 8-byte (u8), 16-byte (u16) or two
-// 16-byte (float) loads and two 16-byte stores where the source row and the
-// destination are aligned for them (checked per pair on the device), scalar
-// accesses otherwise.
 template <typename T>
-__device__ __forceinline__ void ingest_row8(const unsigned char *row, int x, int W, float *d, bool vec)
+__global__ void __launch_bounds__(256) frames_kernel(const FramesArgs a)
 {
-    if (vec && x + 8 <= W) {
-        float v[8];
-        load8<T>(row, x, v);
-        *reinterpret_cast<float4 *>(d) = make_float4(v[0], v[1], v[2], v[3]);
-        *reinterpret_cast<float4 *>(d + 4) = make_float4(v[4], v[5], v[6], v[7]);
-        return;
+    const int pair = blockIdx.z / a.frames, f = blockIdx.z - pair * a.frames;
+    const int x0 = 4 * (blockIdx.x * 32 + (threadIdx.x & 31)), y0 = FR_ROWS * (blockIdx.y * 8 + (threadIdx.x >> 5));
+    if (x0 >= a.W || y0 >= a.H) return;
+    const unsigned char *src = (const unsigned char *)resolve(a.src[f], pair);
+    const bool vec = x0 + 4 <= a.W && ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)a.pitch) & (4 * sizeof(T) - 1)) == 0;
+    float v[FR_ROWS][4];
+#pragma unroll
+    for (int r = 0; r < FR_ROWS; ++r) {
+        const unsigned char *row = src + (long long)min(y0 + r, a.H - 1) * a.pitch;
+        if (vec) {
+            load4<T>(row, x0, v[r]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[r][k] = (float)__ldg(reinterpret_cast<const T *>(row) + min(x0 + k, a.W - 1));
+        }
     }
-    for (int k = 0; k < 8 && x + k < W; ++k) d[k] = (float)__ldg(reinterpret_cast<const T *>(row) + x + k);
+    if (a.ingest && f == 0) {
+        float *d = (float *)resolve(a.full, pair) + (long long)(y0 + a.margin) * a.full_pitch + (x0 + a.margin);
+#pragma unroll
+        for (int r = 0; r < FR_ROWS; ++r)
+            if (y0 + r < a.H) store_run(d + r * a.full_pitch, v[r], a.W - x0);
+    }
+    if (a.levels < 1) return;
+    const int W1 = a.W / 2, H1 = a.H / 2, x1 = x0 / 2, y1 = y0 / 2;
+    float p[FR_ROWS / 2][2];
+#pragma unroll
+    for (int r = 0; r < FR_ROWS / 2; ++r)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            p[r][i] = 0.25f * ((v[2 * r][2 * i] + v[2 * r][2 * i + 1]) + (v[2 * r + 1][2 * i] + v[2 * r + 1][2 * i + 1]));
+    float *d1 = (float *)resolve(a.down[0][f], pair) + (long long)(y1 + a.margin) * a.down_pitch[0] + (x1 + a.margin);
+#pragma unroll
+    for (int r = 0; r < FR_ROWS / 2; ++r)
+        if (y1 + r < H1) store_run(d1 + r * a.down_pitch[0], p[r], W1 - x1);
+    if (a.levels < 2) return;
+    const int W2 = W1 / 2, H2 = H1 / 2, x2 = x1 / 2, y2 = y1 / 2;
+    float *d2 = (float *)resolve(a.down[1][f], pair) + (long long)(y2 + a.margin) * a.down_pitch[1] + (x2 + a.margin);
+#pragma unroll
+    for (int r = 0; r < FR_ROWS / 4; ++r)
+        if (y2 + r < H2 && x2 < W2)
+            d2[r * a.down_pitch[1]] = 0.25f * ((p[2 * r][0] + p[2 * r][1]) + (p[2 * r + 1][0] + p[2 * r + 1][1]));
 }
 
-__global__ void ingest_kernel(const IngestArgs a)
+cudaError_t launch_frames(const FramesArgs &a, int n_pairs, cudaStream_t st)
 {
-    const int pair = blockIdx.z;
-    const int x = 8 * (blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y;
-    if (x >= a.W) return;
-    const unsigned char *src = (const unsigned char *)resolve(a.src, pair);
-    float *dst = (float *)resolve(a.dst, pair);
-    const int bpp = a.fmt == PIX_U8 ? 1 : (a.fmt == PIX_U16 ? 2 : 4);
-    const unsigned char *row = src + (long long)y * a.pitch;
-    float *d = dst + (long long)(y + a.dst_margin) * a.dst_pitch + (x + a.dst_margin);
-    const uintptr_t align = bpp == 1 ? 8 : 16;
-    const bool vec = ((reinterpret_cast<uintptr_t>(row) % align) == 0) && ((reinterpret_cast<uintptr_t>(d) % 16) == 0);
-    if (a.fmt == PIX_U8) ingest_row8<uint8_t>(row, x, a.W, d, vec);
-    else if (a.fmt == PIX_U16) ingest_row8<uint16_t>(row, x, a.W, d, vec);
-    else ingest_row8<float>(row, x, a.W, d, vec);
+    const dim3 grid((a.W + 4 * 32 - 1) / (4 * 32), (a.H + FR_ROWS * 8 - 1) / (FR_ROWS * 8), n_pairs * a.frames);
+    if (a.fmt == PIX_U8) frames_kernel<uint8_t><<<grid, 256, 0, st>>>(a);
+    else if (a.fmt == PIX_U16) frames_kernel<uint16_t><<<grid, 256, 0, st>>>(a);
+    else frames_kernel<float><<<grid, 256, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
 // One CTA copies UPLOAD_ROWS rows of one frame of one pair: 16-byte words
@@ -424,27 +384,6 @@ cudaError_t launch_upload(const UploadArgs &a, int n_pairs, cudaStream_t st)
 {
     dim3 grid((a.H + UPLOAD_ROWS - 1) / UPLOAD_ROWS, 2, n_pairs);
     upload_kernel<<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ingest(const IngestArgs &a, int n_pairs, cudaStream_t st)
-{
-    dim3 grid((a.W + 8 * 128 - 1) / (8 * 128), a.H, n_pairs);
-    ingest_kernel<<<grid, 128, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
-// 256 threads per CTA: up to 128 along a row (four outputs each), the rest
-// over rows
-cudaError_t launch_down(const DownArgs &a, int n_pairs, cudaStream_t st)
-{
-    const int W2 = a.W / 2, H2 = a.H / 2;
-    if (W2 < 1 || H2 < 1) return cudaSuccess;
-    const int quads = (W2 + 3) / 4;
-    const int tx = std::min(128, (quads + 31) / 32 * 32), ty = 256 / tx;
-    dim3 block(tx, ty);
-    dim3 grid((quads + tx - 1) / tx, (H2 + ty - 1) / ty, n_pairs);
-    down_kernel<<<grid, block, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -135,12 +135,21 @@ struct PassArgs {
 // the encoder do not allow them.
 void attach_region_maps(PassArgs &a, int n_pairs);
 
+// A validated field of another grid that a predictor is interpolated from
+// (u.base null: none; per pair, a null entry of a pointer table: none).
+struct FieldSrc {
+    PtrRef u, v;
+    int nx, ny, w, s, levels_up;
+};
+
 struct DeformArgs {
     PtrRef img;
     int fmt;
     long long pitch;       // bytes between image rows
     int W, H;
     PtrRef pred_u, pred_v; // predictor grid (base null: zero displacement)
+    int n_src;             // > 0: the predictor is interpolated from the last of src[0 .. n_src - 1] that
+    FieldSrc src[2];       // the pair has (zero if none) and written to pred_u, pred_v; 0: it is read there
     int w, s, nx, ny;
     float scale;           // 1 (frame B), 0.5 / -0.5 (central warp of B / A)
     int M;                 // margin of the output around the image
@@ -234,29 +243,26 @@ cudaError_t launch_preprocess(const PreArgs &a, void *scratch, cudaStream_t st);
 // state = init ? x : alpha x + (1 - alpha) state, elementwise over n floats.
 cudaError_t launch_ema(const float *x, float *state, size_t n, float alpha, int init, cudaStream_t st);
 
-struct DownArgs {
-    PtrRef src;
+// Float frames of a pair in one launch, each source frame read once: frame A
+// itself in the margin layout (ingest), and up to two 2x2 box levels of the
+// first `frames` of A and B.  A destination holds its interior at (margin,
+// margin) of rows `pitch` floats apart; level l has floor(W / 2^l) x
+// floor(H / 2^l) pixels.
+struct FramesArgs {
+    PtrRef src[2];       // frames A and B
+    int frames;          // 1 or 2
     int fmt;
-    long long pitch;     // bytes
+    long long pitch;     // bytes between source rows
     int W, H;            // source size
-    PtrRef dst;          // float, floor(W/2) x floor(H/2) at (margin, margin) of rows dst_pitch floats apart
-    long long dst_pitch; // floats
-    int dst_margin;
+    int margin;          // of every destination
+    int ingest;          // 1: frame A to full
+    PtrRef full;
+    long long full_pitch;
+    int levels;          // 0, 1 or 2
+    PtrRef down[2][2];   // [level - 1][frame]
+    long long down_pitch[2];
 };
-cudaError_t launch_down(const DownArgs &a, int n_pairs, cudaStream_t st);
-
-// Frame as float into the margin layout (interior only): the correlation
-// pass reads frame A from it.
-struct IngestArgs {
-    PtrRef src;
-    int fmt;
-    long long pitch;     // bytes
-    int W, H;
-    PtrRef dst;
-    long long dst_pitch; // floats
-    int dst_margin;
-};
-cudaError_t launch_ingest(const IngestArgs &a, int n_pairs, cudaStream_t st);
+cudaError_t launch_frames(const FramesArgs &a, int n_pairs, cudaStream_t st);
 
 // Upload of the caller's host frames (page-locked, device-accessible) into the
 // workspace: per pair, frames A and B of H rows of row_bytes, source rows pitch
