@@ -203,7 +203,8 @@ struct rpiv_handle {
     std::map<std::string, cudaGraphExec_t> graphs;
     char *adj_ws = nullptr;
     size_t adj_bytes = 0;
-    float *ref_ws = nullptr;  // refinement: gu, gv, cu, cv (n floats each), score, max|g|
+    float *ref_ws = nullptr;  // refinement: two gradients and two candidate fields (2 n floats each)
+    float *ref_host = nullptr;  // its score and max|g|: page-locked host memory the device writes
     size_t ref_n = 0;
     // stage tracing
     bool tracing = false;
@@ -964,16 +965,12 @@ rpiv_status rpiv_process_pair(rpiv_handle *h, const void *img_a, const void *img
                               cuda_stream);
 }
 
-rpiv_status rpiv_backward(rpiv_handle *h, const void *img_a, const void *img_b, size_t pitch_bytes, const float *u,
-                          const float *v, float grad_score, float *grad_u, float *grad_v, float *score_out,
-                          void *cuda_stream)
+// What rpiv_backward and rpiv_refine check and allocate before their launches on st.
+static rpiv_status begin_adjoint(rpiv_handle *h, size_t pitch_bytes, cudaStream_t st)
 {
-    if (!h || !img_a || !img_b || !u || !v) return fail(RPIV_ERR_INVALID_ARG, "null argument");
-    if ((grad_u == nullptr) != (grad_v == nullptr)) return fail(RPIV_ERR_INVALID_ARG, "grad_u and grad_v: both or neither");
     const size_t bpp = h->cfg.fmt == RPIV_U8 ? 1 : (h->cfg.fmt == RPIV_U16 ? 2 : 4);
     if (pitch_bytes < (size_t)h->cfg.width * bpp || pitch_bytes % bpp)
         return fail(RPIV_ERR_INVALID_ARG, "pitch_bytes smaller than width * bytes per pixel or misaligned");
-    DeviceGuard dg(h->device);
     const StageDef &d = h->stages[h->cfg.predictor_levels];  // first full-resolution pass grid
     const size_t need = adjoint_workspace_bytes(d.W, d.H, d.w, d.s, d.nx, d.ny);
     if (h->adj_bytes < need) {
@@ -989,11 +986,20 @@ rpiv_status rpiv_backward(rpiv_handle *h, const void *img_a, const void *img_b, 
             return fail(RPIV_ERR_OOM, "adjoint workspace allocation failed");
         }
         h->adj_bytes = need;
-        if (poison_scratch() && cudaMemset(h->adj_ws, 0xFF, need) != cudaSuccess)
+        if (poison_scratch() && cudaMemsetAsync(h->adj_ws, 0xFF, need, st) != cudaSuccess)
             return fail(RPIV_ERR_CUDA, "adjoint workspace fill failed");
+        prepare_adjoint();
+        CK(init_adjoint_workspace(h->adj_ws, st), "adjoint workspace initialisation");
     }
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (h->done_recorded) CK(cudaStreamWaitEvent(st, h->done_ev, 0), "ordering wait");
+    return RPIV_OK;
+}
+
+static rpiv_status launch_score(rpiv_handle *h, const void *img_a, const void *img_b, size_t pitch_bytes, const float *u,
+                                const float *v, float grad_score, float *grad_u, float *grad_v, float *score_out,
+                                cudaStream_t st)
+{
+    const StageDef &d = h->stages[h->cfg.predictor_levels];
     AdjArgs a;
     std::memset(&a, 0, sizeof(a));
     a.W = d.W;
@@ -1014,9 +1020,28 @@ rpiv_status rpiv_backward(rpiv_handle *h, const void *img_a, const void *img_b, 
     a.grad_v = grad_v;
     a.score_out = score_out;
     CK(launch_adjoint(a, st), "adjoint launch");
+    return RPIV_OK;
+}
+
+static rpiv_status end_adjoint(rpiv_handle *h, cudaStream_t st)
+{
     CK(cudaEventRecord(h->done_ev, st), "event record");
     h->done_recorded = true;
     return RPIV_OK;
+}
+
+rpiv_status rpiv_backward(rpiv_handle *h, const void *img_a, const void *img_b, size_t pitch_bytes, const float *u,
+                          const float *v, float grad_score, float *grad_u, float *grad_v, float *score_out,
+                          void *cuda_stream)
+{
+    if (!h || !img_a || !img_b || !u || !v) return fail(RPIV_ERR_INVALID_ARG, "null argument");
+    if ((grad_u == nullptr) != (grad_v == nullptr)) return fail(RPIV_ERR_INVALID_ARG, "grad_u and grad_v: both or neither");
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    DeviceGuard dg(h->device);
+    rpiv_status rs = begin_adjoint(h, pitch_bytes, st);
+    if (rs == RPIV_OK)
+        rs = launch_score(h, img_a, img_b, pitch_bytes, u, v, grad_score, grad_u, grad_v, score_out, st);
+    return rs == RPIV_OK ? end_adjoint(h, st) : rs;
 }
 
 rpiv_status rpiv_refine(rpiv_handle *h, const void *img_a, const void *img_b, size_t pitch_bytes, float *u, float *v,
@@ -1027,6 +1052,7 @@ rpiv_status rpiv_refine(rpiv_handle *h, const void *img_a, const void *img_b, si
     DeviceGuard dg(h->device);
     const StageDef &d = h->stages[h->cfg.predictor_levels];
     const size_t n = (size_t)d.nx * d.ny;
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (h->ref_n < n) {
         if (h->ref_ws) {
             cudaDeviceSynchronize();
@@ -1034,47 +1060,65 @@ rpiv_status rpiv_refine(rpiv_handle *h, const void *img_a, const void *img_b, si
             h->ref_ws = nullptr;
             h->ref_n = 0;
         }
-        if (cudaMalloc(&h->ref_ws, sizeof(float) * (4 * n + 64)) != cudaSuccess) {
+        if (cudaMalloc(&h->ref_ws, sizeof(float) * 8 * n) != cudaSuccess) {
             cudaGetLastError();
             return fail(RPIV_ERR_OOM, "refinement buffers allocation failed");
         }
         h->ref_n = n;
     }
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    float *gu = h->ref_ws, *gv = gu + n, *cu = gv + n, *cv = cu + n, *dS = cv + n, *dgmax = dS + 32;
-    auto read = [&](const float *src, float *dst) -> rpiv_status {
-        CK(cudaMemcpyAsync(dst, src, sizeof(float), cudaMemcpyDeviceToHost, st), "score read");
-        CK(cudaStreamSynchronize(st), "score read");
+    if (!h->ref_host && cudaHostAlloc(&h->ref_host, 2 * sizeof(float), cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(RPIV_ERR_OOM, "refinement score allocation failed");
+    }
+    rpiv_status rs = begin_adjoint(h, pitch_bytes, st);
+    if (rs != RPIV_OK) return rs;
+    // The device writes the score into page-locked host memory: a decision
+    // waits for its stream and nothing else.  A candidate's gradient is taken
+    // with its score, since it is the next step's when the candidate is kept
+    // (nearly always); the last step needs none.  One evaluation and one wait
+    // per step, where a score, its gradient and the score once more took two
+    // evaluations and two waits.
+    float *host = h->ref_host, *dhost = nullptr;
+    CK(cudaHostGetDevicePointer(reinterpret_cast<void **>(&dhost), host, 0), "score address");
+    float *grad = h->ref_ws, *next_grad = grad + 2 * n, *cand = grad + 4 * n, *spare = grad + 6 * n;
+    const float *cur_u = u, *cur_v = v;
+    auto finish = [&]() -> rpiv_status {
+        if (cur_u != u) {
+            CK(cudaMemcpyAsync(u, cur_u, sizeof(float) * n, cudaMemcpyDeviceToDevice, st), "result copy");
+            CK(cudaMemcpyAsync(v, cur_v, sizeof(float) * n, cudaMemcpyDeviceToDevice, st), "result copy");
+        }
+        const rpiv_status e = end_adjoint(h, st);
+        if (e != RPIV_OK) return e;
+        CK(cudaStreamSynchronize(st), "result wait");
         return RPIV_OK;
     };
-    rpiv_status rs;
-    float S = 0.f, gmax = 0.f;
-    if ((rs = rpiv_backward(h, img_a, img_b, pitch_bytes, u, v, 1.0f, gu, gv, dS, cuda_stream)) != RPIV_OK) return rs;
-    CK(launch_refine_absmax(gu, gv, (int)n, dgmax, st), "gradient maximum launch");
-    if ((rs = read(dS, &S)) != RPIV_OK || (rs = read(dgmax, &gmax)) != RPIV_OK) return rs;
+    if ((rs = launch_score(h, img_a, img_b, pitch_bytes, u, v, 1.0f, grad, grad + n, dhost, st)) != RPIV_OK) return rs;
+    CK(launch_refine_absmax(grad, grad + n, (int)n, dhost + 1, st), "gradient maximum launch");
+    CK(cudaStreamSynchronize(st), "score read");
+    float S = host[0];
+    const float gmax = host[1];
     if (hist) hist[0] = S;
     for (int k = 0; k < steps; ++k) {
-        if (gmax > 0.f) {
-            double eta = (double)eta0 * std::ldexp(1.0, -k) / (double)gmax;
-            for (int t = 0; t <= halvings; ++t, eta *= 0.5) {
-                CK(launch_refine_axpy(u, v, gu, gv, (float)eta, cu, cv, (int)n, st), "step launch");
-                if ((rs = rpiv_backward(h, img_a, img_b, pitch_bytes, cu, cv, 1.0f, nullptr, nullptr, dS,
-                                        cuda_stream)) != RPIV_OK)
-                    return rs;
-                float Sc = 0.f;
-                if ((rs = read(dS, &Sc)) != RPIV_OK) return rs;
-                if (Sc > S) {
-                    CK(cudaMemcpyAsync(u, cu, sizeof(float) * n, cudaMemcpyDeviceToDevice, st), "step copy");
-                    CK(cudaMemcpyAsync(v, cv, sizeof(float) * n, cudaMemcpyDeviceToDevice, st), "step copy");
-                    break;
-                }
+        double eta = (double)eta0 * std::ldexp(1.0, -k) / (double)gmax;
+        for (int t = 0; gmax > 0.f && t <= halvings; ++t, eta *= 0.5) {
+            CK(launch_refine_axpy(cur_u, cur_v, grad, grad + n, (float)eta, cand, cand + n, (int)n, st), "step launch");
+            float *ng = k + 1 < steps ? next_grad : nullptr;
+            if ((rs = launch_score(h, img_a, img_b, pitch_bytes, cand, cand + n, 1.0f, ng, ng ? ng + n : nullptr, dhost,
+                                   st)) != RPIV_OK)
+                return rs;
+            CK(cudaStreamSynchronize(st), "score read");
+            if (host[0] > S) {
+                S = host[0];
+                cur_u = cand;
+                cur_v = cand + n;
+                std::swap(cand, spare);
+                std::swap(grad, next_grad);
+                break;
             }
         }
-        if ((rs = rpiv_backward(h, img_a, img_b, pitch_bytes, u, v, 1.0f, gu, gv, dS, cuda_stream)) != RPIV_OK)
-            return rs;
-        if ((rs = read(dS, &S)) != RPIV_OK) return rs;
         if (hist) hist[k + 1] = S;
     }
+    if ((rs = finish()) != RPIV_OK) return rs;
     g_err.clear();
     return RPIV_OK;
 }
@@ -1195,6 +1239,7 @@ rpiv_status rpiv_destroy(rpiv_handle *h)
         if (h->ws) cudaFree(h->ws);
         if (h->err_dev) cudaFree(h->err_dev);
         if (h->ref_ws) cudaFree(h->ref_ws);
+        if (h->ref_host) cudaFreeHost(h->ref_host);
         if (h->io_dev) cudaFree(h->io_dev);
         if (h->ring) cudaFreeHost(h->ring);
         if (h->adj_ws) cudaFree(h->adj_ws);

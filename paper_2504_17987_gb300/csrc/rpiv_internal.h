@@ -291,6 +291,10 @@ struct AdjArgs {
 };
 size_t adjoint_workspace_bytes(int W, int H, int w, int s, int nx, int ny);
 cudaError_t launch_adjoint(const AdjArgs &a, cudaStream_t st);
+// Before the first launch on a workspace, on the same stream; and once per
+// device (never inside a stream capture).
+cudaError_t init_adjoint_workspace(void *ws, cudaStream_t st);
+void prepare_adjoint();
 // Refinement step helpers: cu = u + eta gu (and v), and max(|a|, |b|) into *out.
 cudaError_t launch_refine_axpy(const float *u, const float *v, const float *gu, const float *gv, float eta, float *cu,
                                float *cv, int n, cudaStream_t st);
