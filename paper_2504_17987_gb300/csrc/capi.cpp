@@ -199,7 +199,7 @@ struct rpiv_handle {
     // capture streams of the further parts of a split batch, fork and join events
     static constexpr int kParts = 4;
     cudaStream_t cap_part[kParts] = {};
-    cudaEvent_t fork_ev = nullptr, join_ev[kParts] = {};
+    cudaEvent_t fork_ev = nullptr, join_ev[kParts] = {}, upload_ev[kParts] = {};
     std::map<std::string, cudaGraphExec_t> graphs;
     char *adj_ws = nullptr;
     size_t adj_bytes = 0;
@@ -291,9 +291,12 @@ std::string stage_tag(const rpiv_handle *h, const StageDef &d)
 }
 
 // The full schedule for n pairs whose pointers are in h->io_dev.
-// The launch sequence of pairs pair0 .. pair0 + n - 1 of the call.
+// The launch sequence of pairs pair0 .. pair0 + n - 1 of the call.  plan_pairs:
+// the pairs the passes choose between strips and tiles for (0: n).  Uploads
+// (host frames) start once `after` has completed and record `uploaded`.
 rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred, bool any_nopred, cudaStream_t st,
-                             int pair0 = 0)
+                             int pair0 = 0, int plan_pairs = 0, cudaEvent_t after = nullptr,
+                             cudaEvent_t uploaded = nullptr)
 {
     const rpiv_config &c = h->cfg;
     const int L = c.predictor_levels;
@@ -370,6 +373,7 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
         a.out_info = ws(d.off_info);
         a.plan = d.plan;
         a.strip = d.strip;
+        a.plan_pairs = plan_pairs;
         TraceScope ts(h, st, "pass/" + stage_tag(h, d), geom_of(d.W, d.H, d.w, d.s, d.R, d.nx, d.ny, n));
         CK(launch_pass(a, n, st), "correlation pass launch");
         return RPIV_OK;
@@ -429,8 +433,11 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
         ua.dst_pitch = h->in_pitch;
         ua.row_bytes = c.width * (user_fmt == PIX_U8 ? 1 : (user_fmt == PIX_U16 ? 2 : 4));
         ua.H = c.height;
+        ua.beside = uploaded ? 1 : 0;
         TraceScope ts(h, st, "upload", geom_of(c.width, c.height, 0, 0, 0, 0, 0, n));
+        if (after) CK(cudaStreamWaitEvent(st, after, 0), "upload order");
         CK(launch_upload(ua, n, st), "upload launch");
+        if (uploaded) CK(cudaEventRecord(uploaded, st), "upload order");
         img_a = ua.dst_a;
         img_b = ua.dst_b;
         img_pitch = h->in_pitch;
@@ -797,6 +804,9 @@ rpiv_status rpiv_create(const rpiv_config *cfg, int device, rpiv_handle **out)
         if ((e = cudaEventCreateWithFlags(&h->join_ev[i], cudaEventDisableTiming)) != cudaSuccess)
             return cleanup(RPIV_ERR_CUDA, "event creation failed");
     }
+    for (int i = 0; i < rpiv_handle::kParts; ++i)
+        if ((e = cudaEventCreateWithFlags(&h->upload_ev[i], cudaEventDisableTiming)) != cudaSuccess)
+            return cleanup(RPIV_ERR_CUDA, "event creation failed");
     if ((e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming)) != cudaSuccess)
         return cleanup(RPIV_ERR_CUDA, "event creation failed");
     *out = h;
@@ -832,6 +842,33 @@ static int split_parts(int n)
     }
     while (parts > 1 && n / parts < 8) parts /= 2;
     return parts;
+}
+
+struct BatchPart {
+    int first, count, plan_pairs;
+};
+
+// The parts of a captured batch.  With host frames every part is cut once or
+// twice more, and their uploads follow one another, so that all but the first
+// run beside the passes of the parts before (the link, 205 GB/s, takes 41 us for
+// the 8.4 MB of a 2048^2 u8 pair, a quarter of its passes): four such pairs with
+// the 16-bit 16 px pass 792 -> 702 us.  The passes keep the form (strips or tiles) of the
+// uncut parts, and with it their results to the last bit.
+static std::vector<BatchPart> batch_parts(int n, bool host_frames)
+{
+    const int parts = split_parts(n);
+    std::vector<BatchPart> out;
+    for (int i = 0, first = 0; i < parts; ++i) {
+        const int cnt = n / parts + (i < n % parts ? 1 : 0);
+        const int cuts = host_frames ? std::min(cnt, rpiv_handle::kParts / parts) : 1;
+        for (int k = 0, at = first; k < cuts; ++k) {
+            const int c = cnt / cuts + (k < cnt % cuts ? 1 : 0);
+            out.push_back({at, c, cnt});
+            at += c;
+        }
+        first += cnt;
+    }
+    return out;
 }
 
 rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, const void *const *img_b,
@@ -908,30 +945,24 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
         cudaGraph_t graph = nullptr;
         CK(cudaStreamSynchronize(st), "first-run synchronise");
         CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        const int parts = split_parts(n);
-        if (parts > 1) {
-            // independent parts on forked streams of one graph: one part's small
-            // launches and wave tails overlap the others' large passes
-            cudaError_t fe = cudaEventRecord(h->fork_ev, h->cap_stream);
-            int forked = 1;
-            for (; fe == cudaSuccess && forked < parts; ++forked)
-                fe = cudaStreamWaitEvent(h->cap_part[forked], h->fork_ev, 0);
-            if (fe != cudaSuccess) --forked;
-            rs = fe == cudaSuccess ? RPIV_OK : cuda_fail(fe, "capture fork");
-            for (int i = 0, first = 0; i < parts && rs == RPIV_OK; ++i) {
-                const int cnt = n / parts + (i < n % parts ? 1 : 0);
-                rs = enqueue_schedule(h, cnt, pitch_bytes, any_pred, any_nopred, i ? h->cap_part[i] : h->cap_stream,
-                                      first);
-                first += cnt;
-            }
-            // the joins also end the forked streams' parts of the capture on every path
-            for (int i = 1; i < forked; ++i) {
-                cudaError_t je = cudaEventRecord(h->join_ev[i], h->cap_part[i]);
-                if (je == cudaSuccess) je = cudaStreamWaitEvent(h->cap_stream, h->join_ev[i], 0);
-                if (je != cudaSuccess && rs == RPIV_OK) rs = cuda_fail(je, "capture join");
-            }
-        } else {
-            rs = enqueue_schedule(h, n, pitch_bytes, any_pred, any_nopred, h->cap_stream);
+        const std::vector<BatchPart> parts = batch_parts(n, h->cfg.host_frames != 0);
+        const int np = (int)parts.size();
+        // independent parts on forked streams of one graph: one part's small
+        // launches and wave tails overlap the others' large passes
+        cudaError_t fe = np > 1 ? cudaEventRecord(h->fork_ev, h->cap_stream) : cudaSuccess;
+        int forked = 1;
+        for (; fe == cudaSuccess && forked < np; ++forked) fe = cudaStreamWaitEvent(h->cap_part[forked], h->fork_ev, 0);
+        if (fe != cudaSuccess) --forked;
+        rs = fe == cudaSuccess ? RPIV_OK : cuda_fail(fe, "capture fork");
+        for (int i = 0; i < np && rs == RPIV_OK; ++i)
+            rs = enqueue_schedule(h, parts[i].count, pitch_bytes, any_pred, any_nopred, i ? h->cap_part[i] : h->cap_stream,
+                                  parts[i].first, parts[i].plan_pairs, i ? h->upload_ev[i - 1] : nullptr,
+                                  np > 1 ? h->upload_ev[i] : nullptr);
+        // the joins also end the forked streams' parts of the capture on every path
+        for (int i = 1; i < forked; ++i) {
+            cudaError_t je = cudaEventRecord(h->join_ev[i], h->cap_part[i]);
+            if (je == cudaSuccess) je = cudaStreamWaitEvent(h->cap_stream, h->join_ev[i], 0);
+            if (je != cudaSuccess && rs == RPIV_OK) rs = cuda_fail(je, "capture join");
         }
         cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &graph);
         if (rs != RPIV_OK) {
@@ -1235,6 +1266,8 @@ rpiv_status rpiv_destroy(rpiv_handle *h)
             if (h->cap_part[i]) cudaStreamDestroy(h->cap_part[i]);
             if (h->join_ev[i]) cudaEventDestroy(h->join_ev[i]);
         }
+        for (int i = 0; i < rpiv_handle::kParts; ++i)
+            if (h->upload_ev[i]) cudaEventDestroy(h->upload_ev[i]);
         if (h->fork_ev) cudaEventDestroy(h->fork_ev);
         if (h->ws) cudaFree(h->ws);
         if (h->err_dev) cudaFree(h->err_dev);

@@ -355,34 +355,41 @@ cudaError_t launch_frames(const FramesArgs &a, int n_pairs, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// One CTA copies UPLOAD_ROWS rows of one frame of one pair: 16-byte words
-// where the source row starts on a 16-byte boundary, bytes otherwise.
-constexpr int UPLOAD_ROWS = 8;
+// A CTA copies groups of UPLOAD_ROWS rows of one frame of one pair: 16-byte
+// words where the source rows start on 16-byte boundaries, bytes otherwise.
+// Bound by the link to the host (33.5 MB in 163 us, 205 GB/s, as long as
+// cudaMemcpyAsync takes).  Beside other parts' passes about 64 CTAs keep the link
+// 93 % busy; more loads in flight only hold up the passes' own (four 2048^2
+// pairs end to end: 64 CTAs 702 us, 152 714, 304 750, 32 with four loads per
+// thread 717).  Alone, two CTAs per SM.
+constexpr int UPLOAD_ROWS = 8, UPLOAD_CTAS = 64;
 
 __global__ void __launch_bounds__(256) upload_kernel(const UploadArgs a)
 {
     const int pair = blockIdx.z, which = blockIdx.y;
     const unsigned char *src = (const unsigned char *)resolve(which ? a.src_b : a.src_a, pair);
     unsigned char *dst = (unsigned char *)resolve(which ? a.dst_b : a.dst_a, pair);
-    const int nw = a.row_bytes >> 4;
-    for (int r = 0; r < UPLOAD_ROWS; ++r) {
-        const int y = blockIdx.x * UPLOAD_ROWS + r;
-        if (y >= a.H) return;
-        const unsigned char *s = src + (long long)y * a.pitch;
-        unsigned char *d = dst + (long long)y * a.dst_pitch;
-        if (((uintptr_t)s & 15) == 0) {
-            for (int i = threadIdx.x; i < nw; i += blockDim.x)
-                reinterpret_cast<uint4 *>(d)[i] = reinterpret_cast<const uint4 *>(s)[i];
-            for (int i = (nw << 4) + threadIdx.x; i < a.row_bytes; i += blockDim.x) d[i] = s[i];
-        } else {
-            for (int i = threadIdx.x; i < a.row_bytes; i += blockDim.x) d[i] = s[i];
+    const bool words = ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)a.pitch) & 15) == 0;
+    const int nw = words ? a.row_bytes >> 4 : 0, rest = a.row_bytes - (nw << 4);
+    for (int y0 = blockIdx.x * UPLOAD_ROWS; y0 < a.H; y0 += gridDim.x * UPLOAD_ROWS) {
+        const int rows = min(UPLOAD_ROWS, a.H - y0);
+        for (int i = threadIdx.x; i < rows * nw; i += 256) {
+            const int r = i / nw, x = i - r * nw;
+            reinterpret_cast<uint4 *>(dst + (long long)(y0 + r) * a.dst_pitch)[x] =
+                reinterpret_cast<const uint4 *>(src + (long long)(y0 + r) * a.pitch)[x];
+        }
+        for (int i = threadIdx.x; i < rows * rest; i += 256) {
+            const int r = i / rest, x = (nw << 4) + i - r * rest;
+            dst[(long long)(y0 + r) * a.dst_pitch + x] = src[(long long)(y0 + r) * a.pitch + x];
         }
     }
 }
 
 cudaError_t launch_upload(const UploadArgs &a, int n_pairs, cudaStream_t st)
 {
-    dim3 grid((a.H + UPLOAD_ROWS - 1) / UPLOAD_ROWS, 2, n_pairs);
+    const int groups = (a.H + UPLOAD_ROWS - 1) / UPLOAD_ROWS, frames = 2 * n_pairs;
+    const int ctas = a.beside ? UPLOAD_CTAS : 2 * device_sm_count();
+    dim3 grid(std::min(groups, std::max(1, (ctas + frames - 1) / frames)), 2, n_pairs);
     upload_kernel<<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();
 }

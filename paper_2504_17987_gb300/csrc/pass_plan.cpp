@@ -514,11 +514,12 @@ cudaError_t launch_pass(const PassArgs &args_in, int n_pairs, cudaStream_t st)
     PassArgs strip_args;
     if (args_in.strip.strip_rows > 0) {
         // the planned segment length, or shorter segments (down to 2 window
-        // rows) when those give the launch enough CTAs
-        const int ny = args_in.ny;
+        // rows) when those give the launch enough CTAs; a launch cut out of a
+        // larger one (plan_pairs) keeps that one's form, at 2 rows if need be
+        const int ny = args_in.ny, form_pairs = args_in.plan_pairs > 0 ? args_in.plan_pairs : n_pairs;
         for (int L = args_in.strip.strip_rows; L >= 2; L /= 2) {
-            const long long segs = (ny + L - 1) / L;
-            if ((long long)args_in.strip.tiles_x * segs * n_pairs >= strip_min_ctas()) {
+            const long long segs = (ny + L - 1) / L, ctas = args_in.strip.tiles_x * segs;
+            if (ctas * n_pairs >= strip_min_ctas() || (L / 2 < 2 && ctas * form_pairs >= strip_min_ctas())) {
                 strip_args = args_in;
                 strip_args.plan = args_in.strip;
                 strip_args.plan.strip_rows = L;

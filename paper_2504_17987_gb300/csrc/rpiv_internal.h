@@ -124,6 +124,7 @@ struct PassArgs {
     PassPlan plan;
     PassPlan strip;        // strip alternative to the tile plan (strip_rows 0: none); the
                            // launch takes it when the batch gives it enough CTAs
+    int plan_pairs;        // pairs that decision is made for (0: the launch's own)
     // set at launch (attach_region_maps): 3-D tensor maps (column, row, pair)
     // of the A and B' float frames whose boxes are the plan's regions; tma = 0:
     // the regions are loaded row by row
@@ -273,6 +274,7 @@ struct UploadArgs {
     PtrRef dst_a, dst_b;   // workspace frames
     long long dst_pitch;   // bytes between destination rows
     int row_bytes, H;
+    int beside;            // 1: other parts' passes run beside it
 };
 cudaError_t launch_upload(const UploadArgs &a, int n_pairs, cudaStream_t st);
 

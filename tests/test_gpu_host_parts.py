@@ -1,0 +1,39 @@
+"""Captured batches of host frames run in parts whose uploads overlap the passes of
+the parts before: their fields equal a device-frames engine's captured batch bit for
+bit, at part counts of 1 to 4 and in both halves of a split batch, with schedules
+whose strips depend on the number of pairs, and on the eager first call."""
+import pytest
+import torch
+
+import paper_2504_17987_gb300 as rp
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2504_17987_gb300 import build
+    build.build()
+    synth.build()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 16, 19])
+@pytest.mark.parametrize("windows,radii,levels", [((32, 16), (4, 4), 1), ((64, 16), (4, 1), 0)])
+def test_parts_equal_the_uncut_batch(n, windows, radii, levels):
+    W, H = 341, 330  # 341-byte rows: bytes, not words
+    flow = synth.Flow(U=1.3, V=-0.7, vortices=[(0.5 * W, 0.5 * H, 200.0, 20.0)])
+    pairs = [synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=8, ppp=0.05, dp=(2.5, 2.5), seed=300 + k), flow)
+             for k in range(n)]
+    kw = dict(windows=windows, overlaps=(0.5,) * len(windows), radii=radii, levels=levels, max_batch=n)
+    dev, host = rp.Engine(rp.Config(W, H, **kw)), rp.Engine(rp.Config(W, H, host_frames=True, **kw))
+    da, db = [rp.to_device(p[0]) for p in pairs], [rp.to_device(p[1]) for p in pairs]
+    ha, hb = ([rp.to_device(p[k], "cpu", pin=True) for p in pairs] for k in (0, 1))
+    for _ in range(3):  # eager, then captured
+        ref, got = dev.process_batch(da, db), host.process_batch(ha, hb)
+        torch.cuda.synchronize()
+        for x, y in zip(ref, got):
+            assert torch.equal(x, y)
+    host.wait(10000)
+    dev.close()
+    host.close()
