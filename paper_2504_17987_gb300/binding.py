@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import functools
 import os
 from typing import List, Optional, Sequence, Tuple
 
@@ -26,10 +27,11 @@ def _poison() -> bool:
     return os.environ.get("RPIV_POISON_SCRATCH", "") == "1"
 
 
-def _fresh(t: torch.Tensor) -> torch.Tensor:
+def _fresh(*ts: torch.Tensor):
     if _poison():
-        t.view(torch.uint8).fill_(0xFF)
-    return t
+        for t in ts:
+            t.view(torch.uint8).fill_(0xFF)
+    return ts if len(ts) > 1 else ts[0]
 RPIV_FP32, RPIV_BF16, RPIV_FP16 = 0, 1, 2
 RPIV_DEFORM_B, RPIV_DEFORM_CENTRAL = 0, 1
 STATUS = {0: "OK", 1: "INVALID_ARG", 2: "UNSUPPORTED", 3: "OOM", 4: "CUDA", 5: "TIMEOUT", 6: "BUSY", 7: "NO_DEVICE"}
@@ -122,13 +124,19 @@ def _check(st: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# the current stream's handle without a Stream object per call (3 us of a stage call's 12)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch._C._cuda_getDevice())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 @dataclasses.dataclass
@@ -211,6 +219,13 @@ def _entry_ptrs(x, n: int):
     return [x[i].data_ptr() for i in range(n)]
 
 
+@functools.lru_cache(maxsize=64)
+def _dtype_ok(dtype: torch.dtype, cfg_fmt: int) -> bool:
+    if cfg_fmt == RPIV_F32:
+        return dtype == torch.float32
+    return not dtype.is_floating_point and dtype.itemsize == (1 if cfg_fmt == RPIV_U8 else 2)
+
+
 def _img_check(t: torch.Tensor, cfg_fmt: int, host: bool = False):
     if host:
         # that the memory is page-locked is checked by the library, once per
@@ -220,11 +235,7 @@ def _img_check(t: torch.Tensor, cfg_fmt: int, host: bool = False):
             raise ValueError("a host_frames engine takes pinned CPU tensors")
     elif not t.is_cuda:
         raise ValueError("images must be CUDA tensors")
-    if cfg_fmt == RPIV_F32:
-        ok = t.dtype == torch.float32
-    else:
-        ok = not t.is_floating_point() and t.element_size() == (1 if cfg_fmt == RPIV_U8 else 2)
-    if not ok:
+    if not _dtype_ok(t.dtype, cfg_fmt):
         raise ValueError(f"image dtype {t.dtype} does not match the handle's pixel format")
     if t.dim() != 2 or t.stride(1) != 1:
         raise ValueError("images must be 2-D with unit column stride")
@@ -257,6 +268,8 @@ class Engine:
         nx, ny = ctypes.c_int(), ctypes.c_int()
         _check(L.rpiv_grid_shape(h, ctypes.byref(nx), ctypes.byref(ny)))
         self.nx, self.ny = nx.value, ny.value
+        self._dev = torch.device("cuda", device)
+        self._fmt = cfg.fmt
 
     @property
     def handle(self):
@@ -272,15 +285,14 @@ class Engine:
     def empty_outputs(self, n: int = 1):
         """(u, v, vort, mask) for n pairs: u, v and vort are views of one float
         allocation (two allocations instead of four per call)."""
-        dev = torch.device("cuda", self.device)
         shp = (n, self.ny, self.nx) if n > 1 else (self.ny, self.nx)
-        f = torch.empty((3,) + shp, dtype=torch.float32, device=dev)
-        return f[0], f[1], f[2], torch.empty(shp, dtype=torch.uint8, device=dev)
+        u, v, w = torch.empty((3,) + shp, dtype=torch.float32, device=self._dev).unbind(0)
+        return u, v, w, torch.empty(shp, dtype=torch.uint8, device=self._dev)
 
     def process_pair(self, a: torch.Tensor, b: torch.Tensor, pred=None, out=None, stream=None):
         """Returns (u, v, vort, mask) on the final-pass grid (asynchronous)."""
-        _img_check(a, self.cfg.fmt, self.cfg.host_frames)
-        _img_check(b, self.cfg.fmt, self.cfg.host_frames)
+        _img_check(a, self._fmt, self.cfg.host_frames)
+        _img_check(b, self._fmt, self.cfg.host_frames)
         if a.stride(0) != b.stride(0):
             raise ValueError("A and B must share the row pitch")
         u, v, w, m = out if out is not None else self.empty_outputs(1)
@@ -298,7 +310,7 @@ class Engine:
             raise ValueError("a_list and b_list differ in length")
         pitch = a_list[0].stride(0) * a_list[0].element_size()
         for t in list(a_list) + list(b_list):
-            _img_check(t, self.cfg.fmt, self.cfg.host_frames)
+            _img_check(t, self._fmt, self.cfg.host_frames)
             if t.stride(0) * t.element_size() != pitch:
                 raise ValueError("all images of a batch must share the row pitch")
         if outs is None:
@@ -323,8 +335,8 @@ class Engine:
     def score_and_grad(self, a: torch.Tensor, b: torch.Tensor, u: torch.Tensor, v: torch.Tensor,
                        grad_score: float = 1.0, want_grad: bool = True, stream=None):
         """S = sum_w C_w(0) on the first pass's grid and grad_score * dS/d(u, v)."""
-        _img_check(a, self.cfg.fmt)
-        _img_check(b, self.cfg.fmt)
+        _img_check(a, self._fmt)
+        _img_check(b, self._fmt)
         u = u.contiguous().float()
         v = v.contiguous().float()
         dev = u.device
@@ -388,13 +400,14 @@ def stage_correlate(a, b, w: int, s: int, r: int, pred_u=None, pred_v=None, prec
     H, W = a.shape
     nx, ny = (W - w) // s + 1, (H - w) // s + 1
     dev = a.device
-    u = _fresh(torch.empty((ny, nx), dtype=torch.float32, device=dev))
-    v = _fresh(torch.empty_like(u))
-    info = _fresh(torch.empty((ny, nx), dtype=torch.int32, device=dev))
+    u = torch.empty((ny, nx), dtype=torch.float32, device=dev)
+    v = torch.empty_like(u)
+    info = torch.empty((ny, nx), dtype=torch.int32, device=dev)
     dm = RPIV_DEFORM_CENTRAL if deform == "central" else RPIV_DEFORM_B
     nbytes = ctypes.c_size_t()
     _check(load().rpiv_stage_correlate_scratch_bytes(W, H, r, dm, ctypes.byref(nbytes)))
-    scratch = _fresh(torch.empty(max(1, nbytes.value), dtype=torch.uint8, device=dev))
+    scratch = torch.empty(max(1, nbytes.value), dtype=torch.uint8, device=dev)
+    _fresh(u, v, info, scratch)
     _check(load().rpiv_stage_correlate(_ptr(a), _ptr(b), a.stride(0) * a.element_size(), _fmt_code(a), W, H, w, s, r,
                                        PRECISIONS[precision], dm, _ptr(pred_u), _ptr(pred_v), _ptr(u), _ptr(v),
                                        _ptr(info), _ptr(scratch), nbytes.value, _stream(stream)))

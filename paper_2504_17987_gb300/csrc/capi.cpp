@@ -224,7 +224,8 @@ struct DeviceGuard {
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        if (prev != dev) cudaSetDevice(dev);
+        if (prev == dev) prev = -1;  // nothing to put back
+        else cudaSetDevice(dev);
     }
     ~DeviceGuard()
     {

@@ -472,20 +472,48 @@ bool plan_tc(int w, int s, int R, int nx, int ny, PassPlan *plan)
     return true;
 }
 
-bool pass_plan(int w, int s, int R, int nx, int ny, int prec, PassPlan *plan, PassPlan *strip)
+static bool make_plan(int w, int s, int R, int nx, int ny, int prec, bool tc, PassPlan *plan, PassPlan *strip)
 {
     if (w < 2 || s < 1 || nx < 1 || ny < 1 || !pass_supported(R, prec)) return false;
-    if (prec != PREC_FP32 && tc_shape(w, s, R) && tc_planes_enabled()) {
-        if (strip) std::memset(strip, 0, sizeof(*strip));
+    if (tc) {
+        std::memset(strip, 0, sizeof(*strip));
         return plan_tc(w, s, R, nx, ny, plan);
     }
     const int G = gcd(w, s);
     if (prec != PREC_FP32 && (G % 2) != 0) return false;  // paired 16-bit loads need even blocks
-    if (strip) {
-        std::memset(strip, 0, sizeof(*strip));
-        if (!plan_strip(w, s, R, G, nx, ny, prec, strip)) std::memset(strip, 0, sizeof(*strip));
-    }
+    std::memset(strip, 0, sizeof(*strip));
+    if (!plan_strip(w, s, R, G, nx, ny, prec, strip)) std::memset(strip, 0, sizeof(*strip));
     return plan_search(w, s, R, G, nx, ny, prec, plan);
+}
+
+// A plan follows from its arguments alone, and a search takes about 7 us: a
+// stage call, which plans each time, finds the plans of the thread's last few
+// shapes again (a schedule has at most eight).
+bool pass_plan(int w, int s, int R, int nx, int ny, int prec, PassPlan *plan, PassPlan *strip)
+{
+    struct Entry {
+        int key[7];
+        bool used, ok;
+        PassPlan plan, strip;
+    };
+    constexpr int kEntries = 8;
+    static thread_local Entry cache[kEntries] = {};
+    static thread_local int next = 0;
+    const int key[7] = {w, s, R, nx, ny, prec, prec != PREC_FP32 && tc_shape(w, s, R) && tc_planes_enabled() ? 1 : 0};
+    Entry *e = nullptr;
+    for (Entry &c : cache)
+        if (c.used && std::memcmp(c.key, key, sizeof(key)) == 0) e = &c;
+    if (!e) {
+        e = &cache[next];
+        next = (next + 1) % kEntries;
+        std::memcpy(e->key, key, sizeof(key));
+        e->used = true;
+        e->ok = make_plan(w, s, R, nx, ny, prec, key[6] != 0, &e->plan, &e->strip);
+    }
+    if (!e->ok) return false;
+    *plan = e->plan;
+    if (strip) *strip = e->strip;
+    return true;
 }
 
 // A strip launch walks its segments serially inside each CTA, so it is taken
