@@ -355,41 +355,65 @@ cudaError_t launch_frames(const FramesArgs &a, int n_pairs, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// A CTA copies groups of UPLOAD_ROWS rows of one frame of one pair: 16-byte
-// words where the source rows start on 16-byte boundaries, bytes otherwise.
+// A warp copies up to 32 consecutive 16-byte words of a row of one frame of one
+// pair.  Every load is an aligned 16-byte word; where a row starts off a 16-byte
+// boundary, a word of the destination is the end of one and the start of the next,
+// which the next lane holds (the words at a row's ends reach past it, inside the
+// 16 bytes that hold its first or last pixel).
 // Bound by the link to the host (33.5 MB in 163 us, 205 GB/s, as long as
 // cudaMemcpyAsync takes).  Beside other parts' passes about 64 CTAs keep the link
 // 93 % busy; more loads in flight only hold up the passes' own (four 2048^2
 // pairs end to end: 64 CTAs 702 us, 152 714, 304 750, 32 with four loads per
 // thread 717).  Alone, two CTAs per SM.
-constexpr int UPLOAD_ROWS = 8, UPLOAD_CTAS = 64;
+constexpr int UPLOAD_CTAS = 64;
+
+// the 16 bytes from byte sh (0..15) of lo followed by hi
+__device__ __forceinline__ uint4 bytes_from(uint4 lo, uint4 hi, int sh)
+{
+    uint32_t a[7] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z}, last = hi.w;
+    if (sh & 8) {
+        a[0] = a[2], a[1] = a[3], a[2] = a[4], a[3] = a[5], a[4] = a[6], a[5] = last;
+    }
+    if (sh & 4) {
+        a[0] = a[1], a[1] = a[2], a[2] = a[3], a[3] = a[4], a[4] = a[5];
+    }
+    const uint32_t bits = 8u * (sh & 3);
+    return make_uint4(__funnelshift_r(a[0], a[1], bits), __funnelshift_r(a[1], a[2], bits),
+                      __funnelshift_r(a[2], a[3], bits), __funnelshift_r(a[3], a[4], bits));
+}
 
 __global__ void __launch_bounds__(256) upload_kernel(const UploadArgs a)
 {
-    const int pair = blockIdx.z, which = blockIdx.y;
+    const int pair = blockIdx.z, which = blockIdx.y, lane = threadIdx.x & 31;
     const unsigned char *src = (const unsigned char *)resolve(which ? a.src_b : a.src_a, pair);
     unsigned char *dst = (unsigned char *)resolve(which ? a.dst_b : a.dst_a, pair);
-    const bool words = ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)a.pitch) & 15) == 0;
-    const int nw = words ? a.row_bytes >> 4 : 0, rest = a.row_bytes - (nw << 4);
-    for (int y0 = blockIdx.x * UPLOAD_ROWS; y0 < a.H; y0 += gridDim.x * UPLOAD_ROWS) {
-        const int rows = min(UPLOAD_ROWS, a.H - y0);
-        for (int i = threadIdx.x; i < rows * nw; i += 256) {
-            const int r = i / nw, x = i - r * nw;
-            reinterpret_cast<uint4 *>(dst + (long long)(y0 + r) * a.dst_pitch)[x] =
-                reinterpret_cast<const uint4 *>(src + (long long)(y0 + r) * a.pitch)[x];
+    const int nw = (a.row_bytes + 15) >> 4, nc = (nw + 31) >> 5, warps = gridDim.x * 8;
+    for (long long t = blockIdx.x * 8 + (threadIdx.x >> 5); t < (long long)a.H * nc; t += warps) {
+        const int y = (int)(t / nc), x = 32 * (int)(t - (long long)y * nc) + lane;
+        const unsigned char *row = src + (long long)y * a.pitch;
+        const int sh = (int)(reinterpret_cast<uintptr_t>(row) & 15);
+        const uint4 *p = reinterpret_cast<const uint4 *>(row - sh);
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (x < nw) w = p[x];
+        if (sh) {  // the same for the whole warp
+            uint4 n;
+            n.x = __shfl_down_sync(0xffffffffu, w.x, 1);
+            n.y = __shfl_down_sync(0xffffffffu, w.y, 1);
+            n.z = __shfl_down_sync(0xffffffffu, w.z, 1);
+            n.w = __shfl_down_sync(0xffffffffu, w.w, 1);
+            // no next lane holds the following word, and this one needs bytes of it
+            if (x < nw && (lane == 31 || x + 1 == nw) && sh + min(16, a.row_bytes - 16 * x) > 16) n = p[x + 1];
+            w = bytes_from(w, n, sh);
         }
-        for (int i = threadIdx.x; i < rows * rest; i += 256) {
-            const int r = i / rest, x = (nw << 4) + i - r * rest;
-            dst[(long long)(y0 + r) * a.dst_pitch + x] = src[(long long)(y0 + r) * a.pitch + x];
-        }
+        if (x < nw) reinterpret_cast<uint4 *>(dst + (long long)y * a.dst_pitch)[x] = w;
     }
 }
 
 cudaError_t launch_upload(const UploadArgs &a, int n_pairs, cudaStream_t st)
 {
-    const int groups = (a.H + UPLOAD_ROWS - 1) / UPLOAD_ROWS, frames = 2 * n_pairs;
+    const int tasks = a.H * (((a.row_bytes + 15) / 16 + 31) / 32), frames = 2 * n_pairs;
     const int ctas = a.beside ? UPLOAD_CTAS : 2 * device_sm_count();
-    dim3 grid(std::min(groups, std::max(1, (ctas + frames - 1) / frames)), 2, n_pairs);
+    dim3 grid(std::min((tasks + 7) / 8, std::max(1, (ctas + frames - 1) / frames)), 2, n_pairs);
     upload_kernel<<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();
 }

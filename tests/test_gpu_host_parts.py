@@ -21,7 +21,7 @@ def _built():
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 16, 19])
 @pytest.mark.parametrize("windows,radii,levels", [((32, 16), (4, 4), 1), ((64, 16), (4, 1), 0)])
 def test_parts_equal_the_uncut_batch(n, windows, radii, levels):
-    W, H = 341, 330  # 341-byte rows: bytes, not words
+    W, H = 341, 330  # 341-byte rows start anywhere in a 16-byte word
     flow = synth.Flow(U=1.3, V=-0.7, vortices=[(0.5 * W, 0.5 * H, 200.0, 20.0)])
     pairs = [synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=8, ppp=0.05, dp=(2.5, 2.5), seed=300 + k), flow)
              for k in range(n)]
@@ -35,5 +35,30 @@ def test_parts_equal_the_uncut_batch(n, windows, radii, levels):
         for x, y in zip(ref, got):
             assert torch.equal(x, y)
     host.wait(10000)
+    dev.close()
+    host.close()
+
+
+@pytest.mark.parametrize("bits", [8, 12])
+@pytest.mark.parametrize("W", [64, 255, 256, 257, 530, 1029])
+@pytest.mark.parametrize("offset", [0, 1, 3, 13])
+def test_upload_of_rows_at_any_alignment(bits, W, offset):
+    """Rows that start anywhere in a 16-byte word, ragged ends, rows of one to several
+    warps: the fields equal those of the same frames on the device."""
+    H = 72
+    flow = synth.Flow(U=1.3, V=-0.7, vortices=[])
+    A, B = synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=bits, ppp=0.05, dp=(2.5, 2.5), seed=W), flow)
+    kw = dict(windows=(16,), overlaps=(0.5,), radii=(2,), bit_depth=bits)
+    dev, host = rp.Engine(rp.Config(W, H, **kw)), rp.Engine(rp.Config(W, H, host_frames=True, **kw))
+    views = []
+    for img in (A, B):
+        t = rp.to_device(img, "cpu", pin=False)
+        buf = torch.zeros(H, W + offset + 2, dtype=t.dtype).pin_memory()
+        buf[:, offset:offset + W] = t
+        views.append(buf[:, offset:offset + W])
+    ref, got = dev.process_pair(rp.to_device(A), rp.to_device(B)), host.process_pair(*views)
+    torch.cuda.synchronize()
+    for x, y in zip(ref, got):
+        assert torch.equal(x, y)
     dev.close()
     host.close()
