@@ -15,9 +15,10 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(os.path.dirname(HERE), "_build", "rpiv")
 LIB = os.path.join(HERE, "librpiv.so")
 
-SOURCES = ["k_pass_fp32.cu", "k_pass_tc.cu", "k_deform.cu", "k_grid.cu", "k_adjoint.cu",
+SOURCES = ["k_pass_fp32.cu", "k_pass_fp32_r1.cu", "k_pass_fp32_r2.cu", "k_pass_fp32_r4.cu", "k_pass_fp32_r6.cu",
+           "k_pass_fp32_r8.cu", "k_pass_tc.cu", "k_deform.cu", "k_grid.cu", "k_adjoint.cu",
            "k_static_scratch.cu", "k_pre.cu", "pass_plan.cpp", "capi.cpp"]
-HEADERS = ["rpiv_internal.h", "pass_impl.cuh", "tc_pass.cuh", "grid_interp.cuh"]
+HEADERS = ["rpiv_internal.h", "pass_impl.cuh", "pass_fp32.cuh", "tc_pass.cuh", "grid_interp.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", CSRC, "-I", INCLUDE,
            "--expt-relaxed-constexpr"]

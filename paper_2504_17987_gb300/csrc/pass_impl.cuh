@@ -1441,14 +1441,20 @@ static __device__ __forceinline__ void invalid_tile(const PassArgs &a, const Til
 
 // ------------------------------------------------------------- the kernel --
 
+// CTAs per SM a pass kernel is bounded to: those its tiles are planned for
+// (min_ctas in pass_plan.cpp), so that no kernel spills for CTAs its shared memory
+// does not admit; the kernel of any shape serves small windows too.
+constexpr int pass_ctas(int RC, int prec, int GC)
+{
+    if (prec != PREC_FP32 || RC < 0 || RC > 4 || GC >= 24) return 3;
+    if (GC == 8) return RC == 4 ? 3 : 5;
+    return GC > 0 ? 4 : 5;
+}
+
 // GC > 0: a kernel specialised for blocks of GC pixels, windows of 2 GC and
 // steps of GC (50 % overlap), so that window, step and block loops unroll.
-// FP32 kernels up to r = 4 are bounded to five CTAs per SM (48 registers),
-// except the 64 px windows and the 16 px windows at r = 4, whose tiles are
-// planned for three.
 template <int RC, int PREC, int GC>
-__global__ void __launch_bounds__(PASS_THREADS,
-                                  (PREC == PREC_FP32 && (RC >= 0 && RC <= 4) && GC != 32 && !(GC == 8 && RC == 4)) ? 5 : 3)
+__global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     pass_kernel(const __grid_constant__ PassArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
