@@ -357,7 +357,9 @@ __device__ __forceinline__ void tc_copies(const PassArgs &a, const TileGeom &g, 
         const float *br = Bs + ph * P.b_pitch + x;
         uint32_t *d0 = TB0 + ph * hpb + x2, *d1 = TB1 + ph * hpb + x2;
         for (int y = ph; y < g.BR; y += step) {
-            const float v0 = k0 ? br[0] - m : 0.f, v1 = k1 ? br[1] - m : 0.f, v2 = k2 ? br[2] - m : 0.f;
+            // (x, x + 1) by one 8-byte load (x and the pitch are even); columns not staged enter as zeros
+            const float2 f = (k0 || k1) ? *reinterpret_cast<const float2 *>(br) : make_float2(0.f, 0.f);
+            const float v0 = k0 ? f.x - m : 0.f, v1 = k1 ? f.y - m : 0.f, v2 = k2 ? br[2] - m : 0.f;
             *d0 = pack2<PREC>(v0, v1);
             *d1 = pack2<PREC>(v1, v2);
             br += step * P.b_pitch;
@@ -876,6 +878,19 @@ __device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a1,
 
 __device__ __forceinline__ uint32_t ld_pair(const uint16_t *p) { return *reinterpret_cast<const uint32_t *>(p); }
 
+// 8 x 8 blocks of 16-bit values from shared memory, one 16-byte row per lane address
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&d)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x2(uint32_t &d0, uint32_t &d1, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(d0), "=r"(d1) : "r"(addr) : "memory");
+}
+
 // Block planes on the tensor cores, one warp per (block, row group).  For
 // every row r of B' the group meets, the MMA multiplies
 //     X_r[sx][k] = B'[r][x0 + k + sx]        (a Toeplitz matrix of the row: M = sx)
@@ -885,7 +900,10 @@ __device__ __forceinline__ uint32_t ld_pair(const uint16_t *p) { return *reinter
 // directly, for every shift, across the rows.  A rows outside the group come
 // from the zero bands of the slab layout, so every fragment is one load at an
 // offset that only the row step changes.  16 x 8 tiles: MT tiles of sx, NT
-// tiles of sy.
+// tiles of sy.  Where blocks start on 16-byte boundaries of the slabs (G a
+// multiple of 8) the Y fragments of two tiles come from one ldmatrix: they are
+// 8 x 8 blocks of consecutive slab rows (the X rows, shifted by one column each,
+// are not).
 template <int R, int PREC>
 __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeom &g, const uint16_t *TA, const uint16_t *TB,
                                 float *Ps)
@@ -915,9 +933,6 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
         // step t: B' smem row i_lo + 1 + t; lane (n, gq) reads A row i_lo + t - 8 n - gq,
         // i.e. slab row t - 8 n - gq
         const uint16_t *pb = srcB + (i_lo + 1) * bp + colbase + X0;
-        const uint16_t *pa[NT];
-#pragma unroll
-        for (int n = 0; n < NT; ++n) pa[n] = TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * n - gq) * ap + X0 + 2 * tq;
         // the row step advances every fragment pointer by one row
         float acc[MT][NT][4];
 #pragma unroll
@@ -926,16 +941,29 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
             for (int n = 0; n < NT; ++n)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+        // this lane's row address for the Y fragments: lanes 8 i .. 8 i + 7 address the rows of 8 x 8 block i
+        const int mi = lane >> 3, mr = lane & 7;
         if ((G % 16) == 0) {
+            // blocks (n, k half): n + (i >> 1), 8 (i & 1)
+            uint32_t ya = smem_addr(TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * (mi >> 1) - mr) * ap + X0 + 8 * (mi & 1));
 #pragma unroll 2
             for (int t = 0; t < trips; ++t) {
 #pragma unroll
                 for (int X = 0; X < G; X += 16) {
-                    uint32_t bf[NT][2];
+                    uint32_t bf[NT + 1][2];
 #pragma unroll
-                    for (int n = 0; n < NT; ++n) {
-                        bf[n][0] = ld_pair(pa[n] + X);
-                        bf[n][1] = ld_pair(pa[n] + X + 8);
+                    for (int n = 0; n < NT; n += 2) {
+                        uint32_t q[4];
+                        const uint32_t ad = ya + 2 * X - 16 * n * ap;
+                        if (n + 1 < NT) {
+                            ldmatrix_x4(q, ad);
+                            bf[n + 1][0] = q[2];
+                            bf[n + 1][1] = q[3];
+                        } else {
+                            ldmatrix_x2(q[0], q[1], ad);
+                        }
+                        bf[n][0] = q[0];
+                        bf[n][1] = q[1];
                     }
 #pragma unroll
                     for (int m = 0; m < MT; ++m) {
@@ -945,13 +973,31 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
                         for (int n = 0; n < NT; ++n) mma_k16<PREC>(acc[m][n], a0, a1, a1, a3, bf[n][0], bf[n][1]);
                     }
                 }
+                ya += 2 * ap;
+                pb += bp;
+            }
+        } else if (G == 8 && NT == 2) {
+            uint32_t ya = smem_addr(TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * (mi & 1) - mr) * ap + X0);
+#pragma unroll 4
+            for (int t = 0; t < trips; ++t) {
+                uint32_t bf[2];
+                ldmatrix_x2(bf[0], bf[1], ya);
 #pragma unroll
-                for (int n = 0; n < NT; ++n) pa[n] += ap;
+                for (int m = 0; m < MT; ++m) {
+                    const uint16_t *c = pb + 16 * m;
+                    const uint32_t a0 = ld_pair(c), a1 = ld_pair(c + 8);
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) mma_k8<PREC>(acc[m][n], a0, a1, bf[n]);
+                }
+                ya += 2 * ap;
                 pb += bp;
             }
         } else {
-            // G = 8 (or another even size below 16): k8 steps; columns past
+            // other even sizes (and one tile of sy): k8 steps; columns past
             // the block (uneven G) enter as zeros
+            const uint16_t *pa[NT];
+#pragma unroll
+            for (int n = 0; n < NT; ++n) pa[n] = TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * n - gq) * ap + X0 + 2 * tq;
 #pragma unroll 4
             for (int t = 0; t < trips; ++t) {
 #pragma unroll
@@ -1219,17 +1265,19 @@ static __device__ __forceinline__ bool plane_and_peak(const PassArgs &a, const T
     return any_need;
 }
 
-// FP32 planes, compile-time radius: two windows per warp, one per half-warp
+// One plane per block, compile-time radius: two windows per warp, one per half-warp
 // (window 2 pw + h for half h), 16 lanes over the shifts q = lane + 16 j, so
 // that the per-window set-up, reduction and stencil work is shared by two
 // windows.  The half's argmax takes two reductions over its 16 lanes (order
 // key, then q): the largest value, ties to the smallest row-major index, NaN
 // never winning.  Results as plane_and_peak.
-template <int RC>
+// tc: 16-bit planes (moff, and every stencil point by the direct sums), as there.
+template <int RC, bool TC>
 static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, const TileGeom &g, const float *Ps,
                                             const float *Vs, const float *stats, const WinShared &ws,
-                                            int ring_wy = -1)
+                                            float moff = 0.f)
 {
+    constexpr int ring_wy = -1;
     constexpr int R = RC, ND = 2 * RC + 1, NP = ND * ND;
     constexpr int NQ = (NP + 15) / 16;
     constexpr uint32_t NONE = 0xffffffffu;
@@ -1237,10 +1285,14 @@ static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = lane >> 4, hl = lane & 15;
     const int kb = g.kb, sg = g.s / g.G;
-    const int ps = NP, rs = g.nbx * ps;
+    const int ps = TC ? P.pstride : NP, rs = g.nbx * ps;
     const float tau = TAU_PER_PIXEL * (float)(g.w * g.w);
     const int cp = P.v_pitch;
     const float2 *VV = reinterpret_cast<const float2 *>(Vs);
+    const float nm = (float)(g.w * g.w) * moff;
+    auto coef = [&](float num, float muA, float S1, float nB) {
+        return TC ? (num - (muA - moff) * (S1 - nm)) * nB + 0.f : scaled_zncc(num, muA, S1, nB);
+    };
     int qv[NQ], vv[NQ];
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
@@ -1274,7 +1326,7 @@ static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, c
 #pragma unroll
             for (int j = 0; j < NQ; ++j) {
                 if (j < NQ - 1 || hl + 16 * j < NP) {
-                    const float c = scaled_zncc(block_sum(pb, qv[j]), muA, vb[vv[j]].x, vb[vv[j]].y);
+                    const float c = coef(block_sum(pb, qv[j]), muA, vb[vv[j]].x, vb[vv[j]].y);
                     // ascending q: the first of equal values stays; NaN never wins
                     if (c > best || (bq == NONE && c == c)) {
                         best = c;
@@ -1297,7 +1349,7 @@ static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, c
         if (hl < 5 && live) {
             int sy, sx;
             stencil_shift(hl, ky, kx, sy, sx);
-            direct = !(sy >= -R && sy <= R && sx >= -R && sx <= R);
+            direct = TC || !(sy >= -R && sy <= R && sx >= -R && sx <= R);
             if (!direct) {
                 const int q = (sy + R) * ND + (sx + R), vo = sy * cp + sx;
                 c = scaled_zncc(block_sum(pb, q), muA, vb[vo].x, vb[vo].y);
@@ -1318,9 +1370,54 @@ static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, c
 // for the CTA's warps when a tile has fewer windows than warps.
 __device__ __forceinline__ int stencil_groups(int nwin, int w, int nwarps) { return min(max(1, nwarps / nwin), w); }
 
+// All five sums of a row group, W a compile-time window of 16, 32 or 64 px: the
+// lane's pixels e = lane, lane + 32, ... in row-major order, without the walk.
+template <int W>
+__device__ __forceinline__ void stencil_sums(const float *ap, const float *bp, int apt, int bpt, int rows, int lane, float (&acc)[5])
+{
+    constexpr int DY = W < 32 ? 32 / W : 1, NX = W > 32 ? W / 32 : 1;
+    const int y0 = W < 32 ? lane / W : 0, x = W < 32 ? lane & (W - 1) : lane;
+    ap += y0 * apt + x;
+    bp += y0 * bpt + x;
+#pragma unroll 4
+    for (int y = y0; y < rows; y += DY) {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            const float av = ap[32 * k];
+            const float *b = bp + 32 * k;
+            acc[0] = fmaf(av, b[0], acc[0]);
+            acc[1] = fmaf(av, b[-1], acc[1]);
+            acc[2] = fmaf(av, b[1], acc[2]);
+            acc[3] = fmaf(av, b[-bpt], acc[3]);
+            acc[4] = fmaf(av, b[bpt], acc[4]);
+        }
+        ap += DY * apt;
+        bp += DY * bpt;
+    }
+}
+
+// The warp's five sums over its lanes, by the same tree as warp_sum (distances
+// 16, 8, 4, 2, 1), where a lane keeps one of two sums at a step and hands its
+// partner the other: 8 shuffles instead of 25.  The sum of point 0, 1, 2, 3, 4
+// ends in lane 0, 16, 8, 24, 4; the return value is this lane's.
+__device__ __forceinline__ float stencil_reduce(const float (&acc)[5], int lane)
+{
+    auto half = [&](float lo, float hi, int o) {
+        const bool up = lane & o;
+        return (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+    };
+    auto all = [](float v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); };
+    const float p01 = half(acc[0], acc[1], 16), p23 = half(acc[2], acc[3], 16), p4 = all(acc[4], 16);
+    return all(all(half(half(p01, p23, 8), all(p4, 8), 4), 2), 1);
+}
+
 // Direct FP32 numerators of the stencil points the plane cannot supply: one
 // warp per (window, row group), lanes over the group's pixels, five
-// accumulators; dpart[(wi ng + gr) 5 + p] holds a group's partial sum.
+// accumulators; dpart[(wi ng + gr) 5 + p] holds a group's partial sum.  TC: the
+// 16-bit path, where every window needs all five (16 pairs of 1 MP: 64 px 692 ->
+// 656 us, 32 px 487 -> 466, 16 px 549 -> 519 with the wider copies and fragment
+// loads); the FP32 kernels, where few do, keep the shorter code.
+template <bool TC>
 static __device__ __forceinline__ void stencil_direct(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs,
                                       const WinShared &ws)
 {
@@ -1341,7 +1438,13 @@ static __device__ __forceinline__ void stencil_direct(const PassArgs &a, const T
         // B' at A pixel (r, x) and shift (sy, sx): row r + sy + R + 1, column x + sx + padl
         const float *bbase = Bs + (wyi * g.s + r0 + ky + R + 1) * bpt + P.padl + wxi * g.s + kx;
         float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        if (need == 0x1f) {
+        if (TC && need == 0x1f && w == 16) {
+            stencil_sums<16>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
+        } else if (TC && need == 0x1f && w == 32) {
+            stencil_sums<32>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
+        } else if (TC && need == 0x1f && w == 64) {
+            stencil_sums<64>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
+        } else if (need == 0x1f) {
             for (Walk2D e(lane, 32, w); e.y < r1 - r0; e.next()) {
                 const float av = abase[e.y * P.a_pitch + e.x];
                 const float *bb = bbase + e.y * bpt + e.x;
@@ -1361,6 +1464,12 @@ static __device__ __forceinline__ void stencil_direct(const PassArgs &a, const T
                 if (need & 8) acc[3] = fmaf(av, bb[-bpt], acc[3]);
                 if (need & 16) acc[4] = fmaf(av, bb[bpt], acc[4]);
             }
+        }
+        if (TC) {
+            const float v = stencil_reduce(acc, lane);
+            if ((lane & 7) == 0) ws.dpart[it * 5 + ((lane >> 4) | ((lane >> 2) & 2))] = v;
+            else if (lane == 4) ws.dpart[it * 5 + 4] = v;
+            continue;
         }
 #pragma unroll
         for (int p = 0; p < 5; ++p)
@@ -1558,14 +1667,14 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     // tiles: 1.207 -> 1.198 ms per 64-pair launch; with fewer windows the
     // warps left idle cost more than the shared set-up saves)
     bool needs;
-    if (PREC == PREC_FP32 && RC >= 0 && g.nwin >= 2 * (int)(blockDim.x >> 5))
-        needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0)>(a, g, Ps, Vs, stats, ws);
+    if (RC >= 0 && g.nwin >= 2 * (int)(blockDim.x >> 5))
+        needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0), tc>(a, g, Ps, Vs, stats, ws, moff);
     else
         needs = plane_and_peak<RC, PREC == PREC_FP32>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
     // the direct stencil and its barrier only when some window needs them
     // (peaks at the edge of the search, and every window on the 16-bit path)
     if (__syncthreads_or(needs)) {
-        stencil_direct(a, g, As, Bs, ws);
+        stencil_direct<tc>(a, g, As, Bs, ws);
         __syncthreads();
     }
     finalize(a, g, Vs, stats, ws, pair);
@@ -1657,7 +1766,7 @@ __global__ void __launch_bounds__(PASS_THREADS, GC == 32 ? 3 : 4) strip_kernel(c
         // 4: plane, argmax, FP32 stencil, Gaussian fit, outputs
         // the direct stencil and its barrier only when some window needs them
         if (__syncthreads_or(plane_and_peak<RC, true>(a, g, Ps, Vs, stats, false, ws, wy))) {
-            stencil_direct(a, g, As, Bs, ws);
+            stencil_direct<false>(a, g, As, Bs, ws);
             __syncthreads();
         }
         // the regions are read no more in this step: the next step's copies go
