@@ -854,14 +854,18 @@ struct BatchPart {
 // run beside the passes of the parts before (the link, 205 GB/s, takes 41 us for
 // the 8.4 MB of a 2048^2 u8 pair, a quarter of its passes): four such pairs with
 // the 16-bit 16 px pass 792 -> 702 us.  The passes keep the form (strips or tiles) of the
-// uncut parts, and with it their results to the last bit.
-static std::vector<BatchPart> batch_parts(int n, bool host_frames)
+// uncut parts, and with it their results to the last bit.  A part uploads at
+// least 4 MB (20 us): below that the launches it adds cost more than it hides
+// (seven 256 x 1248 u8 pairs, 4.5 MB: four parts 92 us, two 88, one 85).
+static std::vector<BatchPart> batch_parts(int n, size_t upload_bytes_per_pair)
 {
     const int parts = split_parts(n);
+    constexpr size_t kPartBytes = size_t(4) << 20;
     std::vector<BatchPart> out;
     for (int i = 0, first = 0; i < parts; ++i) {
         const int cnt = n / parts + (i < n % parts ? 1 : 0);
-        const int cuts = host_frames ? std::min(cnt, rpiv_handle::kParts / parts) : 1;
+        const int most = (int)std::min<size_t>(rpiv_handle::kParts, upload_bytes_per_pair * cnt / kPartBytes);
+        const int cuts = std::max(1, std::min({cnt, rpiv_handle::kParts / parts, most}));
         for (int k = 0, at = first; k < cuts; ++k) {
             const int c = cnt / cuts + (k < cnt % cuts ? 1 : 0);
             out.push_back({at, c, cnt});
@@ -946,7 +950,7 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
         cudaGraph_t graph = nullptr;
         CK(cudaStreamSynchronize(st), "first-run synchronise");
         CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        const std::vector<BatchPart> parts = batch_parts(n, h->cfg.host_frames != 0);
+        const std::vector<BatchPart> parts = batch_parts(n, h->cfg.host_frames ? 2 * (size_t)h->in_pitch * h->cfg.height : 0);
         const int np = (int)parts.size();
         // independent parts on forked streams of one graph: one part's small
         // launches and wave tails overlap the others' large passes

@@ -2,6 +2,7 @@
 the parts before: their fields equal a device-frames engine's captured batch bit for
 bit, at part counts of 1 to 4 and in both halves of a split batch, with schedules
 whose strips depend on the number of pairs, and on the eager first call."""
+import numpy as np
 import pytest
 import torch
 
@@ -18,13 +19,13 @@ def _built():
     synth.build()
 
 
-@pytest.mark.parametrize("n", [1, 2, 3, 5, 16, 19])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 17])
 @pytest.mark.parametrize("windows,radii,levels", [((32, 16), (4, 4), 1), ((64, 16), (4, 1), 0)])
 def test_parts_equal_the_uncut_batch(n, windows, radii, levels):
-    W, H = 341, 330  # 341-byte rows start anywhere in a 16-byte word
+    W, H = 3341, 630  # 3341-byte rows start anywhere in a 16-byte word; 4.2 MB per pair: one pair per part and more
     flow = synth.Flow(U=1.3, V=-0.7, vortices=[(0.5 * W, 0.5 * H, 200.0, 20.0)])
-    pairs = [synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=8, ppp=0.05, dp=(2.5, 2.5), seed=300 + k), flow)
-             for k in range(n)]
+    base = synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=8, ppp=0.02, dp=(2.5, 2.5), seed=300), flow)
+    pairs = [(np.roll(base[0], 7 * k, 0), np.roll(base[1], 7 * k, 0)) for k in range(n)]
     kw = dict(windows=windows, overlaps=(0.5,) * len(windows), radii=radii, levels=levels, max_batch=n)
     dev, host = rp.Engine(rp.Config(W, H, **kw)), rp.Engine(rp.Config(W, H, host_frames=True, **kw))
     da, db = [rp.to_device(p[0]) for p in pairs], [rp.to_device(p[1]) for p in pairs]
