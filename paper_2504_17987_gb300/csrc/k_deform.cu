@@ -50,17 +50,16 @@ __device__ __forceinline__ void axis_weight(int pos, int n, float c0, int s, int
     t = f - (float)ia;
 }
 
+// Signed integers in the order of the floats they are made of (no NaN), and
+// back: a warp's minimum or maximum is then one reduction instruction.
+__device__ __forceinline__ int order_key(int bits) { return bits ^ ((bits >> 31) & 0x7fffffff); }
 __device__ __forceinline__ float warp_min(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __int_as_float(order_key(__reduce_min_sync(0xffffffffu, order_key(__float_as_int(v)))));
 }
 __device__ __forceinline__ float warp_max(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __int_as_float(order_key(__reduce_max_sync(0xffffffffu, order_key(__float_as_int(v)))));
 }
 
 // A pixel as a float plus the format's bias: integers below 2^23 are placed in
@@ -232,10 +231,14 @@ __device__ void deform_tile(const DeformArgs &a, const unsigned char *img, float
     if (has) {
         int ilo, ihi, jlo, jhi;
         float t;
-        axis_weight(x0, a.nx, c0, a.s, ilo, t);
-        axis_weight(x0 + DTX - 1, a.nx, c0, a.s, ihi, t);
-        axis_weight(y0, a.ny, c0, a.s, jlo, t);
-        axis_weight(y0 + DTY - 1, a.ny, c0, a.s, jhi, t);
+        // the cells of the tile's corners, one per lane
+        const int corner = lane & 3;
+        axis_weight(corner < 2 ? x0 + (corner & 1) * (DTX - 1) : y0 + (corner & 1) * (DTY - 1), corner < 2 ? a.nx : a.ny,
+                    c0, a.s, ilo, t);
+        jhi = __shfl_sync(0xffffffffu, ilo, 3);
+        jlo = __shfl_sync(0xffffffffu, ilo, 2);
+        ihi = __shfl_sync(0xffffffffu, ilo, 1);
+        ilo = __shfl_sync(0xffffffffu, ilo, 0);
         ihi = min(ihi + 1, a.nx - 1);
         jhi = min(jhi + 1, a.ny - 1);
         const int nwn = ihi - ilo + 1, nhn = jhi - jlo + 1;
