@@ -111,7 +111,11 @@ int box_run(int n, int across)
     return 8 * items >= 7 * kThreads ? L : 8;
 }
 
-Layout layout_for(int TX, int TY, int w, int s, int R, int G, int prec, bool strip = false)
+// spread: pitches that keep the two half-warps of the paired peak search in
+// different banks, at some shared memory: planes an odd multiple of 16 floats apart
+// (neighbouring windows' planes then fall 16 banks apart), and rows of V continuing
+// where the shifts of the row before end (2R + 1 pairs, modulo 16).
+Layout layout_for(int TX, int TY, int w, int s, int R, int G, int prec, bool strip = false, bool spread = false)
 {
     PassPlan p;
     std::memset(&p, 0, sizeof(p));
@@ -136,6 +140,8 @@ Layout layout_for(int TX, int TY, int w, int s, int R, int G, int prec, bool str
     p.b_pitch = odd4(p.padl + aw + R + 4);
     p.h_pitch = BC | 1;
     p.v_pitch = (BC - w + 1) | 1;
+    if (spread)
+        while (p.v_pitch % 16 != ND % 16) p.v_pitch += 2;
     p.box_lv = box_run(vh, BC);
     p.box_lh = box_run(BC - w + 1, vh);
     p.box_nv = (vh + p.box_lv - 1) / p.box_lv;
@@ -180,6 +186,7 @@ Layout layout_for(int TX, int TY, int w, int s, int R, int G, int prec, bool str
     const int c_bytes = 2 * vh * p.h_pitch * 4;
     // FP32: one plane per block; TC: the row groups' partial planes, summed in place
     p.pstride = (prec == PREC_FP32 ? 1 : p.RGx) * NP;
+    if (spread) p.pstride = 16 * ((NP + 15) / 16 | 1);
     const int p_bytes = up(nb * p.pstride * 4, 16);
     // direct stencil partials: (window, row group) items, at most max(nwin, warps)
     const int win_bytes = up(nwin * 5 * 4, 16) + up(nwin * 4, 16) * 2 + up(std::max(nwin, kThreads / 32) * 5 * 4, 16);
@@ -384,6 +391,14 @@ bool plan_search(int w, int s, int R, int G, int nx, int ny, int prec, PassPlan 
             }
         }
     if (pick_tx == 0) return false;
+    if (prec == PREC_FP32 && R <= SPREAD_MAX_R && pick_tx * pick_ty >= 2 * kThreads / 32) {
+        // tiles of the paired peak search: spread where it costs no CTA (16 px windows,
+        // r = 4, 64 pairs of 1 MP: 853 -> 824 us).  At r = 6 and 8 tiles seldom have 16
+        // windows, and a stride known only at run time cost 0.5 %.
+        const Layout L = layout_for(pick_tx, pick_ty, w, s, R, G, prec, false, true);
+        auto ctas = [&](int bytes) { return std::min({228 * 1024 / (bytes + 1024), by_regs, by_threads}); };
+        if (L.bytes <= kSmemMax && (!override_kb || L.bytes <= override_kb * 1024) && ctas(L.bytes) >= ctas(pick.bytes)) pick = L;
+    }
     *plan = pick.p;
     plan->tiles_x = (nx + pick_tx - 1) / pick_tx;
     plan->tiles_y = (ny + pick_ty - 1) / pick_ty;

@@ -63,6 +63,10 @@ __device__ __forceinline__ const void *resolve(const PtrRef &r, int pair)
 
 // ------------------------------------------------------------ pass kernel --
 
+// Largest radius whose FP32 tiles may have their planes spread (PassPlan::pstride
+// above the plane's size); beyond it the stride is a constant of the kernel.
+constexpr int SPREAD_MAX_R = 4;
+
 struct PassPlan {
     // tiling
     int TX, TY, tiles_x, tiles_y, threads;
