@@ -286,8 +286,9 @@ class Engine:
         """(u, v, vort, mask) for n pairs: u, v and vort are views of one float
         allocation (two allocations instead of four per call)."""
         shp = (n, self.ny, self.nx) if n > 1 else (self.ny, self.nx)
-        u, v, w = torch.empty((3,) + shp, dtype=torch.float32, device=self._dev).unbind(0)
-        return u, v, w, torch.empty(shp, dtype=torch.uint8, device=self._dev)
+        f = torch.empty((3,) + shp, dtype=torch.float32, device=self._dev)
+        # views of their own: those of one unbind() take no in-place work of an autograd graph
+        return f[0], f[1], f[2], torch.empty(shp, dtype=torch.uint8, device=self._dev)
 
     def process_pair(self, a: torch.Tensor, b: torch.Tensor, pred=None, out=None, stream=None):
         """Returns (u, v, vort, mask) on the final-pass grid (asynchronous)."""
