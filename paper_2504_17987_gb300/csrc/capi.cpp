@@ -7,9 +7,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 #include <map>
 #include <string>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -876,6 +878,31 @@ static std::vector<BatchPart> batch_parts(int n, size_t upload_bytes_per_pair)
     return out;
 }
 
+// Whether a pair's predictor lies in memory that the call writes (a field
+// handed on in place): with parts whose passes follow one another, a later
+// pair would read what an earlier one has written.
+static bool pred_in_outputs(const PairIO *io, int n, size_t count)
+{
+    auto at = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+    std::vector<std::pair<uintptr_t, uintptr_t>> out;
+    for (int i = 0; i < n; ++i) {
+        for (const float *p : {io[i].u, io[i].v, io[i].vort})
+            if (p) out.emplace_back(at(p), at(p) + 4 * count);
+        if (io[i].mask) out.emplace_back(at(io[i].mask), at(io[i].mask) + count);
+    }
+    std::sort(out.begin(), out.end());
+    uintptr_t end = 0;  // running ends: the outputs need not be disjoint
+    for (auto &o : out) o.second = end = std::max(end, o.second);
+    for (int i = 0; i < n; ++i)
+        for (const float *p : {io[i].pred_u, io[i].pred_v}) {
+            if (!p) continue;
+            // the outputs that start before the field's end
+            const auto last = std::lower_bound(out.begin(), out.end(), std::make_pair(at(p) + 4 * count, uintptr_t(0)));
+            if (last != out.begin() && std::prev(last)->second > at(p)) return true;
+        }
+    return false;
+}
+
 rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, const void *const *img_b,
                                size_t pitch_bytes, const float *const *pred_u, const float *const *pred_v,
                                float *const *u, float *const *v, float *const *vort, uint8_t *const *mask,
@@ -934,9 +961,11 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
     CK(cudaMemcpyAsync(h->io_dev, tabh, sizeof(PairIO) * n, cudaMemcpyHostToDevice, st), "pointer table copy");
     CK(cudaEventRecord(h->ring_ev[slot], st), "event record");
     h->ring_used[slot] = true;
-    // launch sequence: captured once per (n, predictor pattern, pitch), then replayed
+    // launch sequence: captured once per (n, predictor pattern, pitch, parts), then replayed
     char keybuf[96];
-    std::snprintf(keybuf, sizeof(keybuf), "%d/%d/%d/%zu", n, (int)any_pred, (int)any_nopred, pitch_bytes);
+    const StageDef &fin = h->stages.back();
+    const bool uncut = !h->cfg.host_frames || (any_pred && pred_in_outputs(tabh, n, (size_t)fin.nx * fin.ny));
+    std::snprintf(keybuf, sizeof(keybuf), "%d/%d/%d/%zu/%d", n, (int)any_pred, (int)any_nopred, pitch_bytes, (int)uncut);
     const std::string key(keybuf);
     auto it = h->graphs.find(key);
     if (h->tracing) {
@@ -950,7 +979,7 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
         cudaGraph_t graph = nullptr;
         CK(cudaStreamSynchronize(st), "first-run synchronise");
         CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        const std::vector<BatchPart> parts = batch_parts(n, h->cfg.host_frames ? 2 * (size_t)h->in_pitch * h->cfg.height : 0);
+        const std::vector<BatchPart> parts = batch_parts(n, uncut ? 0 : 2 * (size_t)h->in_pitch * h->cfg.height);
         const int np = (int)parts.size();
         // independent parts on forked streams of one graph: one part's small
         // launches and wave tails overlap the others' large passes

@@ -360,10 +360,12 @@ int min_ctas(int w, int R, int prec)
 // none fits, the shape with the most CTAs per SM.
 bool plan_search(int w, int s, int R, int G, int nx, int ny, int prec, PassPlan *plan)
 {
-    // registers per thread as the kernels are built: the FP32 kernel is bounded
-    // to five CTAs per SM up to r = 4 (48 registers), three beyond, for the
-    // kernel specialised to 64 px windows at 50 % overlap and for 16 px windows
-    // at r = 4; the tensor-core kernel to three
+    // registers per thread that the search reckons with, from the general FP32
+    // kernel: five CTAs per SM up to r = 4 (48 registers), three beyond, for 64
+    // px windows at 50 % overlap and for 16 px windows at r = 4; the
+    // tensor-core kernel three.  The specialised kernels' own bounds
+    // (pass_ctas) differ for 32 px windows (four); their tiles are kept to this
+    // reckoning, so that a size has the same tiles in either kernel
     const bool wide = (w == 64 && s == 32 && (R == 1 || R == 4)) || (w == 16 && s == 8 && R == 4);
     const int regs = (prec == PREC_FP32 && R <= 4 && !wide) ? 48 : 80;
     const int by_regs = 65536 / (regs * kThreads), by_threads = 2048 / kThreads;

@@ -40,6 +40,32 @@ def test_parts_equal_the_uncut_batch(n, windows, radii, levels):
     host.close()
 
 
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_predictors_in_other_pairs_outputs_are_read_before_they_are_written(shift):
+    """Every pair's predictor is the output memory of another pair (or, shift 0, its own):
+    the fields equal those of a call whose predictors lie elsewhere."""
+    W, H, n = 3341, 630, 4
+    flow = synth.Flow(U=1.3, V=-0.7, vortices=[(0.5 * W, 0.5 * H, 200.0, 20.0)])
+    base = synth.render_pair(synth.ImageSpec(W=W, H=H, bit_depth=8, ppp=0.02, dp=(2.5, 2.5), seed=301), flow)
+    ha, hb = ([rp.to_device(np.roll(base[k], 7 * i, 0), "cpu", pin=True) for i in range(n)] for k in (0, 1))
+    eng = rp.Engine(rp.Config(W, H, windows=(16,), overlaps=(0.5,), radii=(2,), max_batch=n, host_frames=True))
+    fields = [[torch.full((eng.ny, eng.nx), 0.9 + 0.1 * i + 0.05 * k, device="cuda") for k in (0, 1)] for i in range(n)]
+    ref = eng.process_batch(ha, hb, preds=[tuple(f) for f in fields])
+    torch.cuda.synchronize()
+    for _ in range(3):  # eager, then captured
+        outs = eng.empty_outputs(n)
+        for i in range(n):
+            outs[0][i], outs[1][i] = fields[i]
+        preds = [(outs[0][(i + n - shift) % n], outs[1][(i + n - shift) % n]) for i in range(n)]
+        want = ref if not shift else eng.process_batch(ha, hb, preds=[tuple(fields[(i + n - shift) % n]) for i in range(n)])
+        got = eng.process_batch(ha, hb, preds=preds, outs=outs)
+        torch.cuda.synchronize()
+        for x, y in zip(want, got):
+            assert torch.equal(x, y)
+    eng.wait(10000)
+    eng.close()
+
+
 @pytest.mark.parametrize("bits", [8, 12])
 @pytest.mark.parametrize("W", [64, 255, 256, 257, 530, 1029])
 @pytest.mark.parametrize("offset", [0, 1, 3, 13])
