@@ -68,11 +68,11 @@ void attach_region_maps(PassArgs &a, int n_pairs)
     a.tma = 1;
 }
 
-// Radii with a register-blocked fast path (the block size must be a multiple
-// of 4 for its aligned loads); everything else runs the runtime-radius kernel.
+// Radii with a register-blocked fast path; everything else runs the
+// runtime-radius kernel.
 cudaError_t launch_pass_fp32(const PassArgs &a, dim3 grid, int smem, cudaStream_t st)
 {
-    if (a.plan.G % 4 == 0) {
+    if (fp32_radius_kernel(a.R, a.plan.G)) {
         switch (a.R) {
         case 0: return launch_shape<0, 0>(a, grid, smem, st);
         case 1: return launch_radius<1>(a, grid, smem, st);

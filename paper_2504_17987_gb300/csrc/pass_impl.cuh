@@ -1159,7 +1159,8 @@ struct WinShared {
 // step passes the predictor through for them.
 // RC >= 0: compile-time radius; each lane decodes the shifts it owns
 // (q = lane + 32 j) once, into plane and box-sum offsets kept in registers.
-// ONE_PLANE: planes NP floats apart (strips, and tiles whose plan is never spread).
+// ONE_PLANE: planes NP floats apart (strips, and tiles whose plan is never
+// spread); otherwise the plan's stride, which the planes were written at.
 // ring_wy >= 0: strip mode, the window's block rows yy sit in ring rows
 // (ring_wy + yy) & 1.  Returns whether this thread stored a nonzero
 // direct-sum mask (some window needs the direct stencil).
@@ -1670,7 +1671,7 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     if (RC >= 0 && g.nwin >= 2 * (int)(blockDim.x >> 5))
         needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0), tc>(a, g, Ps, Vs, stats, ws, moff);
     else
-        needs = plane_and_peak<RC, PREC == PREC_FP32 && (RC < 0 || RC > SPREAD_MAX_R)>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
+        needs = plane_and_peak<RC, PREC == PREC_FP32 && (RC > SPREAD_MAX_R)>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
     // the direct stencil and its barrier only when some window needs them
     // (peaks at the edge of the search, and every window on the 16-bit path)
     if (__syncthreads_or(needs)) {

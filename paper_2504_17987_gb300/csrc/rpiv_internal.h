@@ -63,8 +63,14 @@ __device__ __forceinline__ const void *resolve(const PtrRef &r, int pair)
 
 // ------------------------------------------------------------ pass kernel --
 
+// Whether an FP32 pass of radius R on blocks of G px runs a kernel with a
+// compile-time radius (its aligned loads want blocks that are a multiple of 4);
+// the kernel of any radius serves the rest.  Read by the dispatch and by the planner.
+constexpr bool fp32_radius_kernel(int R, int G) { return G % 4 == 0 && ((R >= 0 && R <= 4) || R == 6 || R == 8); }
+
 // Largest radius whose FP32 tiles may have their planes spread (PassPlan::pstride
-// above the plane's size); beyond it the stride is a constant of the kernel.
+// above the plane's size); the kernels of larger compile-time radii hold the
+// stride as a constant.
 constexpr int SPREAD_MAX_R = 4;
 
 struct PassPlan {
