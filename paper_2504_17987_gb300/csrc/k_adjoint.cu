@@ -172,7 +172,7 @@ __host__ __device__ inline BlockGrid block_grid(int w, int s, int nx, int ny)
 constexpr int WIN_CTA = 64;      // windows per CTA of adj_windows, WIN_LANES threads each
 constexpr int WIN_LANES = 4;
 constexpr int MAX_G = 32;        // blocks of adj_blocks
-constexpr int NODE_SMEM = 160 * 1024;  // most shared memory of adj_nodes
+constexpr int NODE_SMEM = 192 * 1024;  // most shared memory of adj_nodes
 constexpr int TILE_W = 64, TILE_H = 32;  // its tile is about TILE_W x TILE_H pixels, whole blocks
 
 inline int win_ctas(int nx, int ny) { return (nx * ny + WIN_CTA - 1) / WIN_CTA; }
@@ -219,8 +219,9 @@ NodeTile node_tile(int W, int H, int w, int s, int nx, int ny)
     t.bw = t.rw / G + 2;
     t.bh = t.rh / G + 2;
     // coefficients, the region's products (odd pitch), row sums, the axes' cells, weights and blocks
-    const long long bytes = 4ll * (5ll * t.bw * t.bh + 2ll * t.rh * (t.rw | 1) + 2ll * t.rh * t.tx + 3ll * t.rw + 3ll * t.rh);
-    t.ok = bytes <= NODE_SMEM;
+    const long long nblk = (long long)t.bw * t.bh;
+    const long long bytes = 4ll * (6ll * nblk + 2ll * t.rh * (t.rw | 1) + 2ll * t.rh * t.tx + 3ll * t.rw + 3ll * t.rh);
+    t.ok = bytes - 4ll * nblk <= 160 * 1024;  // so bytes <= NODE_SMEM: nblk takes at least 20 of the bytes on the left
     t.smem = t.ok ? (int)bytes : 0;
     return t;
 }
@@ -524,42 +525,62 @@ __global__ void __launch_bounds__(WIN_CTA *WIN_LANES) adj_windows(const AdjArgs 
     if (threadIdx.x == 0) *ws.ticket = 0u;
 }
 
-// sum over a block's windows of the coefficients of dC_w/dB' = (A - mean A_w) rs_w
-// - (B' - mean B'_w) q_w, with the pixel values taken relative to the block's
-// means: x P - y Q - K with x = A - mA, y = B' - mB, P = sum rs_w, Q = sum q_w.
-// Where the frames correlate the two products nearly cancel, and a rounding of
-// P is common to all of a block's pixels, which the sums over nodes do not
-// average out.  So the difference is formed first: e P + y D - K with
-// e = (A - B') - (mA - mB) and D = sum (rs_w - q_w), K alike (gradient error
-// against 64 bits, 1024^2 u8, 32 px at 75 %: 2.7e-7 -> 2.2e-7).
-// (the window rows from j0, every dj-th)
-__device__ __forceinline__ void block_coefs(const AdjArgs &a, const AdjWs &ws, const BlockGrid &bg, int bx, int by, int j0,
-                                            int dj, float4 &c, float &K)
+// sum over a block's windows of dC_w/dB' = (A - mean A_w) rs_w - (B' - mean B'_w) q_w
+// (rs_w = 1/sqrt(E_A E_B), q_w = C_w/E_B).  Where the frames correlate the two products
+// nearly cancel, and a rounding of the sums P = sum rs_w or Q = sum q_w is common to all
+// of a block's pixels, which the sums over nodes do not average out.  So the difference
+// is formed first: e P + y D - K with e = (A - rA) - rho B', y = B' - mB (the block's
+// mean), D = sum (rho rs_w - q_w) and K the same with the windows' means.
+//   rho  the gain q / rs of the middle window (its regression of A on B'; 0: it has none),
+//   rA   the frames' offset mA - rho mB, cut to 12 bits so that A - rA is exact for integers;
+// every term is then about as small as the result, whatever the contrasts and offsets of
+// the frames are (256^2, 32 px at 75 %, error against 64 bits with B k times as bright:
+// 2.2e-7 at every k, 2.2e-7 with A raised by 1000; with the plain difference A - B' it was
+// 2.2e-7, 4.4e-7 at k = 4, 3.3e-5 at k = 255, and 6.7e-7 for the raised A).  P is the
+// middle window's rs as often as there are windows, plus the sum of the small
+// differences, which rounds once.
+// LANES threads (a power of two, neighbours) share a block, every LANES-th window row
+// each, and all of them must call.
+struct BlockCoefs {
+    float rA, mB, rho, P, D, K;
+};
+
+template <int LANES>
+__device__ __forceinline__ BlockCoefs block_coefs(const AdjArgs &a, const AdjWs &ws, const BlockGrid &bg, int bx, int by)
 {
-    const int w = a.w, s = a.s;
+    const int w = a.w, s = a.s, l = LANES > 1 ? threadIdx.x & (LANES - 1) : 0;
     // G divides w and s, so that indices are those of blocks (usually s = G)
     const int kb = w / bg.G, ks = s / bg.G;
     const int ilo = max(0, ks == 1 ? bx - kb + 1 : (bx - kb + ks) / ks), ihi = min(a.nx - 1, ks == 1 ? bx : bx / ks);
     const int jlo = max(0, ks == 1 ? by - kb + 1 : (by - kb + ks) / ks), jhi = min(a.ny - 1, ks == 1 ? by : by / ks);
     const float4 b = ws.blk[by * bg.nbx + bx];
-    const float e0 = b.x - b.y;
-    float P = 0.f, D = 0.f;
-    K = 0.f;
-    for (int j = jlo + j0; j <= jhi; j += dj)
+    // every block of the windows' union lies in a window (s <= w): ilo <= ihi, jlo <= jhi
+    const float4 m = ws.win4[((jlo + jhi) >> 1) * a.nx + ((ilo + ihi) >> 1)];
+    BlockCoefs r{0.f, b.y, m.z > 0.f ? __fdividef(m.w, m.z) : 0.f, 0.f, 0.f, 0.f};  // rho need not be exact
+    r.rA = __uint_as_float(__float_as_uint(fmaf(-r.rho, b.y, b.x)) & 0xfffff000u);
+    for (int j = jlo + l; j <= jhi; j += LANES)
 #pragma unroll 4
         for (int i = ilo; i <= ihi; ++i) {
             const float4 t = ws.win4[j * a.nx + i];
-            const float d = t.z - t.w;
-            P += t.z;
-            D += d;
-            K = fmaf((t.x - t.y) - e0, t.z, fmaf(t.y - b.y, d, K));
+            const float d = fmaf(r.rho, t.z, -t.w);
+            r.P += t.z - m.z;
+            r.D += d;
+            r.K = fmaf(fmaf(-r.rho, t.y, t.x - r.rA), t.z, fmaf(t.y - b.y, d, r.K));
         }
-    c = make_float4(e0, b.y, P, D);
+#pragma unroll
+    for (int o = 1; o < LANES; o <<= 1) {
+        r.P += __shfl_xor_sync(0xffffffffu, r.P, o);
+        r.D += __shfl_xor_sync(0xffffffffu, r.D, o);
+        r.K += __shfl_xor_sync(0xffffffffu, r.K, o);
+    }
+    r.P = fmaf((float)((ihi - ilo + 1) * (jhi - jlo + 1)), m.z, r.P);
+    return r;
 }
 
-__device__ __forceinline__ float pixel_g(float4 v, float4 c, float K)
+// a pixel (B', grad B, A) of the block
+__device__ __forceinline__ float pixel_g(float4 v, const BlockCoefs &c)
 {
-    return fmaf((v.w - v.x) - c.x, c.z, fmaf(v.x - c.y, c.w, -K));
+    return fmaf(fmaf(-c.rho, v.x, v.w - c.rA), c.P, fmaf(v.x - c.mB, c.D, -c.K));
 }
 
 // 3: one tile of nodes per CTA.  Its region (the union of the nodes' supports)
@@ -570,13 +591,13 @@ __global__ void __launch_bounds__(256) adj_nodes(const AdjArgs a, const AdjWs ws
 {
     extern __shared__ float4 smem4[];
     const int pitch = t.rw | 1;
-    float4 *coef = smem4;                                              // bw x bh
-    float2 *gxy = reinterpret_cast<float2 *>(coef + t.bw * t.bh);      // region, odd pitch
+    float4 *coef = smem4;                                              // bw x bh: rA, mB, rho, P
+    float2 *coef2 = reinterpret_cast<float2 *>(coef + t.bw * t.bh);    // bw x bh: D, K
+    float2 *gxy = coef2 + t.bw * t.bh;                                 // region, odd pitch
     float2 *rows = gxy + t.rh * pitch;                                 // rh x tx
     int2 *cw = reinterpret_cast<int2 *>(rows + t.rh * t.tx);           // per column: node cell and weight
     int2 *rw_ = cw + t.rw;                                             // per row
-    float *coefk = reinterpret_cast<float *>(rw_ + t.rh);              // bw x bh
-    int *cb = reinterpret_cast<int *>(coefk + t.bw * t.bh);            // blocks of the columns and rows
+    int *cb = reinterpret_cast<int *>(rw_ + t.rh);                     // blocks of the columns and rows
     int *rb = cb + t.rw;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = bg.G;
     const float c0 = 0.5f * (float)(a.w - 1);
@@ -609,18 +630,10 @@ __global__ void __launch_bounds__(256) adj_nodes(const AdjArgs a, const AdjWs ws
     for (int by = warp; by < bh; by += 8)
         for (int b8 = 0; b8 < bw; b8 += 8) {
             const int bx = b8 + (lane >> 2);
-            float4 c;
-            float K;
-            block_coefs(a, ws, bg, bx0 + min(bx, bw - 1), by0 + by, lane & 3, 4, c, K);
-#pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
-                c.z += __shfl_xor_sync(0xffffffffu, c.z, o);
-                c.w += __shfl_xor_sync(0xffffffffu, c.w, o);
-                K += __shfl_xor_sync(0xffffffffu, K, o);
-            }
+            const BlockCoefs c = block_coefs<4>(a, ws, bg, bx0 + min(bx, bw - 1), by0 + by);
             if ((lane & 3) == 0 && bx < bw) {
-                coef[by * t.bw + bx] = c;
-                coefk[by * t.bw + bx] = K;
+                coef[by * t.bw + bx] = make_float4(c.rA, c.mB, c.rho, c.P);
+                coef2[by * t.bw + bx] = make_float2(c.D, c.K);
             }
         }
     __syncthreads();
@@ -642,7 +655,9 @@ __global__ void __launch_bounds__(256) adj_nodes(const AdjArgs a, const AdjWs ws
                 const int y = y0 + 8 * r;
                 if (y >= rh) break;
                 const int k = rb[y] + col;
-                const float g = x < xe && y < ye ? pixel_g(v[r], coef[k], coefk[k]) : 0.f;
+                const float4 c = coef[k];
+                const float2 d = coef2[k];
+                const float g = x < xe && y < ye ? pixel_g(v[r], BlockCoefs{c.x, c.y, c.z, c.w, d.x, d.y}) : 0.f;
                 gxy[y * pitch + x] = make_float2(g * v[r].y, g * v[r].z);
             }
         }
@@ -693,11 +708,8 @@ __global__ void adj_pix_kernel(const AdjArgs a, const AdjWs ws, const BlockGrid 
     const long long p = (long long)y * a.W + x;
     float2 g = make_float2(0.f, 0.f);
     if (x < bg.nbx * bg.G && y < bg.nby * bg.G) {
-        float4 c;
-        float K;
-        block_coefs(a, ws, bg, x / bg.G, y / bg.G, 0, 1, c, K);
         const float4 v = ws.px4[p];
-        const float d = pixel_g(v, c, K);
+        const float d = pixel_g(v, block_coefs<1>(a, ws, bg, x / bg.G, y / bg.G));
         g = make_float2(d * v.y, d * v.z);
     }
     ws.pix_g[p] = g;
