@@ -174,6 +174,17 @@ constexpr int kRing = 16;
 
 }  // namespace
 
+struct BatchPart {
+    int first, count, plan_pairs;
+};
+
+// A batch shape's captured sequences: its parts, and the launch sequence in
+// parts (exec[0]) and in one (exec[1], calls whose parts would conflict).
+struct BatchGraphs {
+    std::vector<BatchPart> parts;
+    cudaGraphExec_t exec[2] = {};
+};
+
 struct rpiv_handle {
     rpiv_config cfg{};
     int device = 0;
@@ -202,7 +213,7 @@ struct rpiv_handle {
     static constexpr int kParts = 4;
     cudaStream_t cap_part[kParts] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kParts] = {}, upload_ev[kParts] = {};
-    std::map<std::string, cudaGraphExec_t> graphs;
+    std::map<std::string, BatchGraphs> graphs;
     char *adj_ws = nullptr;
     size_t adj_bytes = 0;
     float *ref_ws = nullptr;  // refinement: two gradients and two candidate fields (2 n floats each)
@@ -847,10 +858,6 @@ static int split_parts(int n)
     return parts;
 }
 
-struct BatchPart {
-    int first, count, plan_pairs;
-};
-
 // The parts of a captured batch.  With host frames every part is cut once or
 // twice more, and their uploads follow one another, so that all but the first
 // run beside the passes of the parts before (the link, 205 GB/s, takes 41 us for
@@ -878,28 +885,35 @@ static std::vector<BatchPart> batch_parts(int n, size_t upload_bytes_per_pair)
     return out;
 }
 
-// Whether a pair's predictor lies in memory that the call writes (a field
-// handed on in place): with parts whose passes follow one another, a later
-// pair would read what an earlier one has written.
-static bool pred_in_outputs(const PairIO *io, int n, size_t count)
+// Whether a pair's predictor lies in memory that the call writes for a pair of
+// another part (a field handed on in place): the parts run side by side or one
+// after another, so it could be read after it is written.  Inside a part every
+// predictor is read before any field is written.
+static bool parts_conflict(const PairIO *io, const std::vector<BatchPart> &parts, size_t count)
 {
     auto at = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
     std::vector<std::pair<uintptr_t, uintptr_t>> out;
-    for (int i = 0; i < n; ++i) {
-        for (const float *p : {io[i].u, io[i].v, io[i].vort})
-            if (p) out.emplace_back(at(p), at(p) + 4 * count);
-        if (io[i].mask) out.emplace_back(at(io[i].mask), at(io[i].mask) + count);
-    }
-    std::sort(out.begin(), out.end());
-    uintptr_t end = 0;  // running ends: the outputs need not be disjoint
-    for (auto &o : out) o.second = end = std::max(end, o.second);
-    for (int i = 0; i < n; ++i)
-        for (const float *p : {io[i].pred_u, io[i].pred_v}) {
-            if (!p) continue;
-            // the outputs that start before the field's end
-            const auto last = std::lower_bound(out.begin(), out.end(), std::make_pair(at(p) + 4 * count, uintptr_t(0)));
-            if (last != out.begin() && std::prev(last)->second > at(p)) return true;
+    for (const BatchPart &w : parts) {
+        out.clear();
+        for (const PairIO *p = io + w.first; p < io + w.first + w.count; ++p) {
+            for (const float *f : {p->u, p->v, p->vort})
+                if (f) out.emplace_back(at(f), at(f) + 4 * count);
+            if (p->mask) out.emplace_back(at(p->mask), at(p->mask) + count);
         }
+        std::sort(out.begin(), out.end());
+        uintptr_t end = 0;  // running ends: the outputs need not be disjoint
+        for (auto &o : out) o.second = end = std::max(end, o.second);
+        for (const BatchPart &r : parts) {
+            if (r.first == w.first) continue;
+            for (const PairIO *p = io + r.first; p < io + r.first + r.count; ++p)
+                for (const float *f : {p->pred_u, p->pred_v}) {
+                    if (!f) continue;
+                    // the outputs that start before the field's end
+                    const auto last = std::lower_bound(out.begin(), out.end(), std::make_pair(at(f) + 4 * count, uintptr_t(0)));
+                    if (last != out.begin() && std::prev(last)->second > at(f)) return true;
+                }
+        }
+    }
     return false;
 }
 
@@ -961,17 +975,19 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
     CK(cudaMemcpyAsync(h->io_dev, tabh, sizeof(PairIO) * n, cudaMemcpyHostToDevice, st), "pointer table copy");
     CK(cudaEventRecord(h->ring_ev[slot], st), "event record");
     h->ring_used[slot] = true;
-    // launch sequence: captured once per (n, predictor pattern, pitch, parts), then replayed
+    // launch sequence: captured once per (n, predictor pattern, pitch, whether
+    // its parts conflict), then replayed
     char keybuf[96];
     const StageDef &fin = h->stages.back();
-    const bool uncut = !h->cfg.host_frames || (any_pred && pred_in_outputs(tabh, n, (size_t)fin.nx * fin.ny));
-    std::snprintf(keybuf, sizeof(keybuf), "%d/%d/%d/%zu/%d", n, (int)any_pred, (int)any_nopred, pitch_bytes, (int)uncut);
-    const std::string key(keybuf);
-    auto it = h->graphs.find(key);
+    std::snprintf(keybuf, sizeof(keybuf), "%d/%d/%d/%zu", n, (int)any_pred, (int)any_nopred, pitch_bytes);
+    BatchGraphs &g = h->graphs[keybuf];
+    if (g.parts.empty()) g.parts = batch_parts(n, h->cfg.host_frames ? 2 * (size_t)h->in_pitch * h->cfg.height : 0);
+    const bool whole = g.parts.size() > 1 && any_pred && parts_conflict(tabh, g.parts, (size_t)fin.nx * fin.ny);
+    cudaGraphExec_t &exec = g.exec[whole ? 1 : 0];
     if (h->tracing) {
         rpiv_status rs = enqueue_schedule(h, n, pitch_bytes, any_pred, any_nopred, st);
         if (rs != RPIV_OK) return rs;
-    } else if (it == h->graphs.end()) {
+    } else if (!exec) {
         // first use of this shape: run eagerly, then capture the same sequence
         // on the handle's private stream for later replays
         rpiv_status rs = enqueue_schedule(h, n, pitch_bytes, any_pred, any_nopred, st);
@@ -979,7 +995,7 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
         cudaGraph_t graph = nullptr;
         CK(cudaStreamSynchronize(st), "first-run synchronise");
         CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        const std::vector<BatchPart> parts = batch_parts(n, uncut ? 0 : 2 * (size_t)h->in_pitch * h->cfg.height);
+        const std::vector<BatchPart> parts = whole ? std::vector<BatchPart>{{0, n, n}} : g.parts;
         const int np = (int)parts.size();
         // independent parts on forked streams of one graph: one part's small
         // launches and wave tails overlap the others' large passes
@@ -1004,13 +1020,14 @@ rpiv_status rpiv_process_batch(rpiv_handle *h, int n, const void *const *img_a, 
             return rs;
         }
         if (ce != cudaSuccess) return cuda_fail(ce, "end capture");
-        cudaGraphExec_t exec = nullptr;
         ce = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
-        if (ce != cudaSuccess) return cuda_fail(ce, "graph instantiate");
-        h->graphs[key] = exec;
+        if (ce != cudaSuccess) {
+            exec = nullptr;
+            return cuda_fail(ce, "graph instantiate");
+        }
     } else {
-        CK(cudaGraphLaunch(it->second, st), "graph launch");
+        CK(cudaGraphLaunch(exec, st), "graph launch");
     }
     CK(cudaEventRecord(h->done_ev, st), "event record");
     h->done_recorded = true;
@@ -1286,7 +1303,9 @@ rpiv_status rpiv_destroy(rpiv_handle *h)
     {
         DeviceGuard dg(h->device);
         if (h->done_ev && h->done_recorded) cudaEventSynchronize(h->done_ev);
-        for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second);
+        for (auto &kv : h->graphs)
+            for (cudaGraphExec_t e : kv.second.exec)
+                if (e) cudaGraphExecDestroy(e);
         for (auto &t : h->trace_evs) {
             cudaEventDestroy(t.t0);
             cudaEventDestroy(t.t1);
