@@ -844,18 +844,14 @@ rpiv_status rpiv_workspace_bytes(const rpiv_handle *h, size_t *bytes)
 }
 
 // Captured batches of 16 pairs and more run as parts of at least 8 pairs on
-// forked streams, two by default (RPIV_SPLIT_BATCH = 1, 2 or 4 parts; read
-// when a batch shape is captured).  Measured on the 64-pair 1 MP workload:
+// forked streams, two by default (RPIV_SPLIT_BATCH = 2 or 4 parts, 0 or 1: none;
+// read when a batch shape is first used).  Measured on the 64-pair 1 MP workload:
 // one chain 13420, two parts 13664-13690, four parts 13346 pairs/s.
-static int split_parts(int n)
+static int most_parts()
 {
-    int parts = 2;
-    if (const char *e = std::getenv("RPIV_SPLIT_BATCH")) {
-        const int v = std::atoi(e);
-        parts = (v == 1 || v == 2 || v == 4) ? v : (v == 0 ? 1 : 2);
-    }
-    while (parts > 1 && n / parts < 8) parts /= 2;
-    return parts;
+    const char *e = std::getenv("RPIV_SPLIT_BATCH");
+    const int v = e ? std::atoi(e) : 2;
+    return (v == 0 || v == 1) ? 1 : (v == 4 ? 4 : 2);
 }
 
 // The parts of a captured batch.  With host frames every part is cut once or
@@ -866,9 +862,13 @@ static int split_parts(int n)
 // uncut parts, and with it their results to the last bit.  A part uploads at
 // least 4 MB (20 us): below that the launches it adds cost more than it hides
 // (seven 256 x 1248 u8 pairs, 4.5 MB: four parts 92 us, two 88, one 85).
+// Where parts are turned off the batch stays in one.
 static std::vector<BatchPart> batch_parts(int n, size_t upload_bytes_per_pair)
 {
-    const int parts = split_parts(n);
+    const int allowed = most_parts();
+    if (allowed == 1) return {{0, n, n}};
+    int parts = allowed;
+    while (parts > 1 && n / parts < 8) parts /= 2;
     constexpr size_t kPartBytes = size_t(4) << 20;
     std::vector<BatchPart> out;
     for (int i = 0, first = 0; i < parts; ++i) {

@@ -47,3 +47,10 @@ def test_calls_whose_parts_do_not_conflict_stay_in_parts(probe, host):
     for shift in (-1, 0):
         res = probe("".join(f"batch {FRAMES[host]} {n} {host} {shift}\n" for n in (1, 4, 16, 33)))
         assert [r[:2] for r in res] == [[0, p] for p in ((1, 4, 4, 4) if host else (1, 1, 2, 2))]
+
+
+@pytest.mark.parametrize("setting", ["0", "1"])
+def test_parts_can_be_turned_off(probe, setting):
+    text = "".join(f"batch {FRAMES[host]} {n} {host} -1\n" for host in (0, 1) for n in (4, 16, 33))
+    assert [r[1] for r in probe(text, {"RPIV_SPLIT_BATCH": setting})] == [1] * 6
+    assert [r[1] for r in probe(text, {"RPIV_SPLIT_BATCH": "4"})] == [1, 2, 4, 4, 4, 4]
