@@ -1067,11 +1067,15 @@ static rpiv_status begin_adjoint(rpiv_handle *h, size_t pitch_bytes, cudaStream_
             cudaGetLastError();
             return fail(RPIV_ERR_OOM, "adjoint workspace allocation failed");
         }
-        h->adj_bytes = need;
-        if (poison_scratch() && cudaMemsetAsync(h->adj_ws, 0xFF, need, st) != cudaSuccess)
-            return fail(RPIV_ERR_CUDA, "adjoint workspace fill failed");
         prepare_adjoint();
-        CK(init_adjoint_workspace(h->adj_ws, st), "adjoint workspace initialisation");
+        cudaError_t e = poison_scratch() ? cudaMemsetAsync(h->adj_ws, 0xFF, need, st) : cudaSuccess;
+        if (e == cudaSuccess) e = init_adjoint_workspace(h->adj_ws, st);
+        if (e != cudaSuccess) {  // not kept: the next call makes and initialises another
+            cudaFree(h->adj_ws);
+            h->adj_ws = nullptr;
+            return cuda_fail(e, "adjoint workspace initialisation");
+        }
+        h->adj_bytes = need;
     }
     if (h->done_recorded) CK(cudaStreamWaitEvent(st, h->done_ev, 0), "ordering wait");
     return RPIV_OK;

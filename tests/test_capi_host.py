@@ -54,3 +54,9 @@ def test_parts_can_be_turned_off(probe, setting):
     text = "".join(f"batch {FRAMES[host]} {n} {host} -1\n" for host in (0, 1) for n in (4, 16, 33))
     assert [r[1] for r in probe(text, {"RPIV_SPLIT_BATCH": setting})] == [1] * 6
     assert [r[1] for r in probe(text, {"RPIV_SPLIT_BATCH": "4"})] == [1, 2, 4, 4, 4, 4]
+
+
+def test_a_score_workspace_that_could_not_be_initialised_is_not_used(probe):
+    # three calls, the first one's initialisation fails (status CUDA); per call: status,
+    # initialisations done, evaluations launched
+    assert probe("adjoint\n") == [[4, 0, 0, 0, 1, 1, 0, 1, 2]]
