@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(256) adj_blocks(const AdjArgs a, const AdjWs w
     }
 }
 
-// 1, blocks above MAX_G and steps below 3 px: the pixels, then one warp per block
+// 1, blocks above MAX_G and steps below 3 px: the pixels, then the blocks
 template <typename T>
 __global__ void adj_deform_kernel(const AdjArgs a, const AdjWs ws)
 {
@@ -394,35 +394,57 @@ __global__ void adj_deform_kernel(const AdjArgs a, const AdjWs ws)
     ws.px4[(long long)y * a.W + x] = make_float4(b, gx, gy, px<T>(A, a.pitch, x, y));
 }
 
-__global__ void adj_block_kernel(const AdjArgs a, const AdjWs ws, const BlockGrid bg)
+// WARPS warps per block: one, or eight for blocks above MAX_G, which are few and have
+// thousands of pixels each (score of a 1 MP pair: 128 px windows without overlap, 64
+// blocks, 229 -> 50 us; 64 px, 256 blocks, 73 -> 26 us).
+template <int WARPS>
+__global__ void __launch_bounds__(256) adj_block_kernel(const AdjArgs a, const AdjWs ws, const BlockGrid bg)
 {
-    const int lane = threadIdx.x & 31;
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (b >= bg.nbx * bg.nby) return;
+    __shared__ float part[5][WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, own = WARPS > 1 ? warp : 0;
+    const int b = WARPS > 1 ? (int)blockIdx.x : (int)blockIdx.x * 8 + warp;
+    if (b >= bg.nbx * bg.nby) return;  // (one warp per block only)
+    // sum k of the warp, and, after a barrier, of the block's warps
+    auto put = [&](float v, int k) {
+        v = wsum(v);
+        if (WARPS > 1 && lane == 0) part[k][own] = v;
+        return v;
+    };
+    auto get = [&](float v, int k) {
+        if (WARPS == 1) return v;
+        float s = 0.f;
+        for (int i = 0; i < WARPS; ++i) s += part[k][i];
+        return s;
+    };
     const int by = b / bg.nbx, bx = b - by * bg.nbx;
     const int G = bg.G, n = G * G;
     const float4 *p = ws.px4 + (long long)(by * G) * a.W + bx * G;
+    const int start = own * 32 + lane;
     float sa = 0.f, sb = 0.f;
-    for (Walk e(lane, 32, G); e.y < G; e.next()) {
+    for (Walk e(start, 32 * WARPS, G); e.y < G; e.next()) {
         const float4 v = p[(long long)e.y * a.W + e.x];
         sa += v.w;
         sb += v.x;
     }
-    const float ma = wsum(sa) / (float)n, mb = wsum(sb) / (float)n;
+    sa = put(sa, 0);
+    sb = put(sb, 1);
+    if (WARPS > 1) __syncthreads();
+    const float ma = get(sa, 0) / (float)n, mb = get(sb, 1) / (float)n;
     float caa = 0.f, cbb = 0.f, cab = 0.f;
-    for (Walk e(lane, 32, G); e.y < G; e.next()) {
+    for (Walk e(start, 32 * WARPS, G); e.y < G; e.next()) {
         const float4 v = p[(long long)e.y * a.W + e.x];
         const float at = v.w - ma, bt = v.x - mb;
         caa = fmaf(at, at, caa);
         cbb = fmaf(bt, bt, cbb);
         cab = fmaf(at, bt, cab);
     }
-    caa = wsum(caa);
-    cbb = wsum(cbb);
-    cab = wsum(cab);
-    if (lane == 0) {
-        ws.blk[b] = make_float4(ma, mb, caa, cbb);
-        ws.blk_ab[b] = cab;
+    caa = put(caa, 2);
+    cbb = put(cbb, 3);
+    cab = put(cab, 4);
+    if (WARPS > 1) __syncthreads();
+    if (lane == 0 && own == 0) {
+        ws.blk[b] = make_float4(ma, mb, get(caa, 2), get(cbb, 3));
+        ws.blk_ab[b] = get(cab, 4);
     }
 }
 
@@ -802,7 +824,8 @@ cudaError_t run(const AdjArgs &a, cudaStream_t st)
         else adj_blocks<T, false><<<grid, 256, 0, st>>>(a, ws, bg, tbx, tby, lanes);
     } else {
         adj_deform_kernel<T><<<dim3((a.W + 255) / 256, a.H), 256, 0, st>>>(a, ws);
-        adj_block_kernel<<<(nblk * 32 + 255) / 256, 256, 0, st>>>(a, ws, bg);
+        if (bg.G > MAX_G) adj_block_kernel<8><<<nblk, 256, 0, st>>>(a, ws, bg);
+        else adj_block_kernel<1><<<(nblk + 7) / 8, 256, 0, st>>>(a, ws, bg);
     }
     const NodeTile t = node_tile(a.W, a.H, a.w, a.s, a.nx, a.ny);
     const int wc = win_ctas(a.nx, a.ny);
