@@ -36,6 +36,7 @@ constexpr int PRE_THREADS = 256;
 constexpr int BATCH = 8;        // rows of vertical sums staged at a time
 constexpr int STRIP = 256;      // columns staged at a time
 constexpr int CHUNK = 512;      // widest chunk
+constexpr int FILTER_COLS = 128;  // widest chunk without equalisation
 constexpr int COPIES = 16;      // copies of a chunk's histogram
 constexpr int MAX_HP = 64;      // largest box radius
 constexpr int RUN = 4;          // consecutive pixels per thread: the horizontal sum slides along them
@@ -46,8 +47,8 @@ __device__ __forceinline__ int px(const unsigned char *img, long long pitch, int
     return (int)__ldg(reinterpret_cast<const T *>(img + (long long)y * pitch) + x);
 }
 
-// Chunks: every tile of the histogram grid is cut into ncx x ncy chunks of
-// cw x ch pixels (the last ones smaller, possibly empty).
+// Chunks: every tile of the histogram grid (without equalisation: the frame) is cut
+// into ncx x ncy chunks of cw x ch pixels (the last ones smaller, possibly empty).
 struct PreSplit {
     int tw, th, ncx, ncy, cw, ch;
     long long bin_pitch;  // bytes between rows of the bins, a multiple of 4
@@ -259,34 +260,45 @@ __global__ void __launch_bounds__(PRE_THREADS) clahe_apply(const PreArgs a, cons
 
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Chunks of about 16 rows and at most CHUNK columns, none below 512 pixels
+// With equalisation: chunks of about 16 rows and at most CHUNK columns, none below 512 pixels
 // unless it is a whole tile: the partial histograms (1 KB each) then fit the
 // first scratch frame (4 bytes per pixel); if rounding up the tiles of an odd
 // size says otherwise, one chunk per tile, whose counts sit where its map goes.
+// Without: the tiles mean nothing, and the frame is cut into chunks of at most
+// FILTER_COLS columns and 16 rows (391 x 277 u8, radius 64: cut by 64 x 64 tiles
+// it took 41 us, by one tile 38, now 14: the host).
 PreSplit split_tiles(const PreArgs &a)
 {
     PreSplit q;
+    q.bin_pitch = (a.W + 3) / 4 * 4;
+    if (a.clip_pct <= 0) {
+        q.tw = a.W;
+        q.th = a.H;
+        q.ncx = (a.W + FILTER_COLS - 1) / FILTER_COLS;
+        q.cw = (a.W + q.ncx - 1) / q.ncx;
+        q.ch = 16;
+        q.ncy = (a.H + q.ch - 1) / q.ch;
+        return q;
+    }
     q.tw = (a.W + a.tx - 1) / a.tx;
     q.th = (a.H + a.ty - 1) / a.ty;
     q.ncx = (q.tw + CHUNK - 1) / CHUNK;
     q.cw = (q.tw + q.ncx - 1) / q.ncx;
     const int rows = std::max(16, (CHUNK + q.cw - 1) / q.cw);
     q.ncy = std::max(1, q.th / rows);
-    if (a.clip_pct > 0 && (size_t)a.tx * a.ty * q.ncx * q.ncy * NBINS * 4 > up256((size_t)a.W * a.H * 4)) {
+    if ((size_t)a.tx * a.ty * q.ncx * q.ncy * NBINS * 4 > up256((size_t)a.W * a.H * 4)) {
         q.ncx = q.ncy = 1;
         q.cw = q.tw;
     }
     q.ch = (q.th + q.ncy - 1) / q.ncy;
-    q.bin_pitch = (a.W + 3) / 4 * 4;
     return q;
 }
 
 template <typename T>
 void launch_bins(const PreArgs &a, const PreSplit &q, uint8_t *bins, int *parts, cudaStream_t st)
 {
-    const dim3 grid(a.tx * q.ncx, a.ty * q.ncy);
-    if (a.clip_pct > 0) pre_bins<T, true><<<grid, PRE_THREADS, 0, st>>>(a, q, bins, parts);
-    else pre_bins<T, false><<<grid, PRE_THREADS, 0, st>>>(a, q, bins, parts);
+    if (a.clip_pct > 0) pre_bins<T, true><<<dim3(a.tx * q.ncx, a.ty * q.ncy), PRE_THREADS, 0, st>>>(a, q, bins, parts);
+    else pre_bins<T, false><<<dim3(q.ncx, q.ncy), PRE_THREADS, 0, st>>>(a, q, bins, parts);
 }
 
 }  // namespace
