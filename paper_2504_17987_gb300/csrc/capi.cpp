@@ -447,7 +447,7 @@ rpiv_status enqueue_schedule(rpiv_handle *h, int n, size_t pitch, bool any_pred,
         ua.dst_pitch = h->in_pitch;
         ua.row_bytes = c.width * (user_fmt == PIX_U8 ? 1 : (user_fmt == PIX_U16 ? 2 : 4));
         ua.H = c.height;
-        ua.beside = uploaded ? 1 : 0;
+        ua.beside = after ? 1 : 0;  // the first part's has the device to itself
         TraceScope ts(h, st, "upload", geom_of(c.width, c.height, 0, 0, 0, 0, 0, n));
         if (after) CK(cudaStreamWaitEvent(st, after, 0), "upload order");
         CK(launch_upload(ua, n, st), "upload launch");

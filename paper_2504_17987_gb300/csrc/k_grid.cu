@@ -364,7 +364,8 @@ cudaError_t launch_frames(const FramesArgs &a, int n_pairs, cudaStream_t st)
 // cudaMemcpyAsync takes).  Beside other parts' passes about 64 CTAs keep the link
 // 93 % busy; more loads in flight only hold up the passes' own (four 2048^2
 // pairs end to end: 64 CTAs 702 us, 152 714, 304 750, 32 with four loads per
-// thread 717).  Alone, two CTAs per SM.
+// thread 717).  Alone, as the first part's is, two CTAs per SM (17 pairs of 407 x 297
+// u16 and 64 CTAs for the first part too: 118 us, 110 before the parts).
 constexpr int UPLOAD_CTAS = 64;
 
 // the 16 bytes from byte sh (0..15) of lo followed by hi

@@ -4,8 +4,9 @@
 // come before each, so that a captured batch's order can be checked.  Commands on stdin:
 //   batch W H n host shift   a process_batch whose predictors are pair (i + shift) mod n's
 //                            outputs (shift -1: other memory), run twice;
-//                            prints "status parts unordered": the parts of the captured
-//                            sequence and the (read, write) pairs it leaves unordered
+//                            prints "status parts unordered beside": the parts of the captured
+//                            sequence, the (read, write) pairs it leaves unordered and the
+//                            uploads that are launched as running beside other parts' passes
 //   adjoint                  score calls of which the first one's initialisation of the
 //                            workspace fails; prints per call "status initialised launched"
 #include <bitset>
@@ -53,7 +54,7 @@ std::map<cudaStream_t, Set> at;
 std::map<cudaEvent_t, Set> ev;
 const PairIO *io_base = nullptr;
 size_t handles = 0;
-int inits = 0, fail_inits = 0, adjoints = 0;
+int inits = 0, fail_inits = 0, adjoints = 0, beside = 0;
 
 int pair_of(const PtrRef &r) { return (int)((r.base - reinterpret_cast<const char *>(io_base)) / (long long)sizeof(PairIO)); }
 
@@ -86,7 +87,11 @@ cudaError_t launch_uod(const UodArgs &a, int n, cudaStream_t st)
 }
 cudaError_t launch_vort(const VortArgs &a, int n, cudaStream_t st) { return op(st, false, true, pair_of(a.u), n); }
 cudaError_t launch_frames(const FramesArgs &, int, cudaStream_t st) { return op(st, false, false, 0, 0); }
-cudaError_t launch_upload(const UploadArgs &, int, cudaStream_t st) { return op(st, false, false, 0, 0); }
+cudaError_t launch_upload(const UploadArgs &a, int, cudaStream_t st)
+{
+    beside += a.beside;
+    return op(st, false, false, 0, 0);
+}
 cudaError_t launch_interp(const InterpArgs &, int, cudaStream_t st) { return op(st, false, false, 0, 0); }
 cudaError_t launch_preprocess(const PreArgs &, void *, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_ema(const float *, float *, size_t, float, int, cudaStream_t) { return cudaSuccess; }
@@ -157,6 +162,7 @@ cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *t, cudaEvent_t, cudaEvent_t) { return *t = 0.f, cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode)
 {
+    beside = 0;
     ops.clear();
     at.clear();
     ev.clear();
@@ -214,7 +220,7 @@ static void batch(int W, int H, int n, int host, int shift)
             unordered += shared;
         }
     }
-    std::printf("%d %d %d\n", (int)st, (int)parts.size(), unordered);
+    std::printf("%d %d %d %d\n", (int)st, (int)parts.size(), unordered, beside);
     rpiv_destroy(h);
 }
 

@@ -35,7 +35,7 @@ FRAMES = {0: "256 256", 1: "3341 630"}  # host frames: 4.2 MB per pair, a part e
 def test_predictors_in_other_parts_outputs_are_read_before_they_are_written(probe, n, host):
     shifts = sorted({0, 1, n // 2, n - 1})
     res = probe("".join(f"batch {FRAMES[host]} {n} {host} {k}\n" for k in shifts))
-    for shift, (status, parts, unordered) in zip(shifts, res):
+    for shift, (status, parts, unordered, _) in zip(shifts, res):
         assert status == 0 and unordered == 0, (shift, parts)
         if shift and n > 1 and (host or n >= 16):
             assert parts == 1  # some pair's predictor lies in another part's outputs
@@ -60,3 +60,9 @@ def test_a_score_workspace_that_could_not_be_initialised_is_not_used(probe):
     # three calls, the first one's initialisation fails (status CUDA); per call: status,
     # initialisations done, evaluations launched
     assert probe("adjoint\n") == [[4, 0, 0, 0, 1, 1, 0, 1, 2]]
+
+
+def test_only_later_parts_uploads_make_room_for_passes(probe):
+    # the first part's upload runs before any pass, with the device to itself
+    res = probe("".join(f"batch {FRAMES[1]} {n} 1 -1\n" for n in (1, 2, 4, 33)))
+    assert [r[3] for r in res] == [r[1] - 1 for r in res] == [0, 1, 3, 3]
