@@ -6,7 +6,7 @@
 
 namespace rpiv {
 
-template <int PREC, int RC, int GC = 0>
+template <int PREC, int RC, int GC = BLOCKS_ANY>
 static cudaError_t go_mma(const PassArgs &a, dim3 grid, int smem, cudaStream_t st)
 {
     pass_kernel<RC, PREC, GC><<<grid, PASS_THREADS, smem, st>>>(a);
@@ -18,6 +18,14 @@ static cudaError_t go_tcgen05(const PassArgs &a, dim3 grid, int smem, cudaStream
 {
     tc_pass_kernel<PREC, GC><<<grid, PASS_THREADS, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+// no kernel specialised to the block size
+template <int PREC, int RC>
+static cudaError_t go_blocks(const PassArgs &a, dim3 grid, int smem, cudaStream_t st)
+{
+    if (tc_slab_blocks(RC, a.plan.G)) return go_mma<PREC, RC, BLOCKS_SLAB>(a, grid, smem, st);
+    return go_mma<PREC, RC, BLOCKS_ANY>(a, grid, smem, st);
 }
 
 // 50 % overlap with 8-, 16- and 32-px blocks at r = 4: the tcgen05 kernel when
@@ -38,7 +46,7 @@ static cudaError_t go_r4(const PassArgs &a, dim3 grid, int smem, cudaStream_t st
         if (G == 16) return go_mma<PREC, 4, 16>(a, grid, smem, st);
         if (G == 32) return go_mma<PREC, 4, 32>(a, grid, smem, st);
     }
-    return go_mma<PREC, 4>(a, grid, smem, st);
+    return go_blocks<PREC, 4>(a, grid, smem, st);
 }
 
 template <int PREC>
@@ -48,8 +56,8 @@ static cudaError_t launch_16bit(const PassArgs &a, dim3 grid, int smem, cudaStre
     case 1: return go_mma<PREC, 1>(a, grid, smem, st);
     case 2: return go_mma<PREC, 2>(a, grid, smem, st);
     case 4: return go_r4<PREC>(a, grid, smem, st);
-    case 6: return go_mma<PREC, 6>(a, grid, smem, st);
-    case 8: return go_mma<PREC, 8>(a, grid, smem, st);
+    case 6: return go_blocks<PREC, 6>(a, grid, smem, st);
+    case 8: return go_blocks<PREC, 8>(a, grid, smem, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -80,6 +88,9 @@ static void prepare_16bit()
     set_smem(pass_kernel<4, PREC, 0>);
     set_smem(pass_kernel<6, PREC, 0>);
     set_smem(pass_kernel<8, PREC, 0>);
+    set_smem(pass_kernel<4, PREC, BLOCKS_SLAB>);
+    set_smem(pass_kernel<6, PREC, BLOCKS_SLAB>);
+    set_smem(pass_kernel<8, PREC, BLOCKS_SLAB>);
     set_smem(pass_kernel<4, PREC, 8>);
     set_smem(pass_kernel<4, PREC, 16>);
     set_smem(pass_kernel<4, PREC, 32>);

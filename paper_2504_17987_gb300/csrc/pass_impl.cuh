@@ -891,6 +891,16 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t &d0, uint32_t &d1, uint32_t
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(d0), "=r"(d1) : "r"(addr) : "memory");
 }
 
+// The 16-bit kernels that are not specialised to one block size (GC <= 0).  Up to r = 2
+// one serves them all; from r = 4 on, where registers are short, one serves the blocks
+// whose Y fragments come by ldmatrix (BLOCKS_SLAB) and one the rest (BLOCKS_ANY), without
+// unrolled stencils or pairs of windows beyond r = 4.  As one kernel the code of the other
+// sizes spilled and cost the rest 1 to 3.5 % (16 pairs of 1 MP, r = 6: 24 px at 50 % 1122
+// us, 12 px 1990; as two 1086 and 1861; 32 px, of the slab blocks, 922 -> 759).
+constexpr int BLOCKS_ANY = 0, BLOCKS_SLAB = -1;
+constexpr bool tc_split(int R) { return R >= 4; }
+constexpr bool tc_slab_blocks(int R, int G) { return G % 16 == 0 || (G == 8 && (2 * R + 8) / 8 == 2); }
+
 // Block planes on the tensor cores, one warp per (block, row group).  For
 // every row r of B' the group meets, the MMA multiplies
 //     X_r[sx][k] = B'[r][x0 + k + sx]        (a Toeplitz matrix of the row: M = sx)
@@ -904,7 +914,7 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t &d0, uint32_t &d1, uint32_t
 // multiple of 8) the Y fragments of two tiles come from one ldmatrix: they are
 // 8 x 8 blocks of consecutive slab rows (the X rows, shifted by one column each,
 // are not).
-template <int R, int PREC>
+template <int R, int PREC, int GC>
 __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeom &g, const uint16_t *TA, const uint16_t *TB,
                                 float *Ps)
 {
@@ -912,6 +922,7 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
     constexpr int NP = ND * ND;
     constexpr int MT = (ND + 15) / 16;
     constexpr int NT = (ND + 7) / 8;
+    constexpr bool SLAB = GC != BLOCKS_ANY || !tc_split(R), REST = GC != BLOCKS_SLAB;  // block sizes the kernel meets
     const PassPlan &P = a.plan;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int gq = lane >> 2, tq = lane & 3;
@@ -943,12 +954,12 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
                 for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
         // this lane's row address for the Y fragments: lanes 8 i .. 8 i + 7 address the rows of 8 x 8 block i
         const int mi = lane >> 3, mr = lane & 7;
-        if ((G % 16) == 0) {
+        if (SLAB && (G % 16) == 0) {
             // blocks (n, k half): n + (i >> 1), 8 (i & 1)
             uint32_t ya = smem_addr(TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * (mi >> 1) - mr) * ap + X0 + 8 * (mi & 1));
 #pragma unroll 2
             for (int t = 0; t < trips; ++t) {
-#pragma unroll
+#pragma unroll (GC == BLOCKS_SLAB ? 1 : 8)
                 for (int X = 0; X < G; X += 16) {
                     uint32_t bf[NT + 1][2];
 #pragma unroll
@@ -976,7 +987,7 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
                 ya += 2 * ap;
                 pb += bp;
             }
-        } else if (G == 8 && NT == 2) {
+        } else if (SLAB && NT == 2 && (!REST || G == 8)) {
             uint32_t ya = smem_addr(TA + (tc_slab_row(R, rows, byi * RG + gi) - 8 * (mi & 1) - mr) * ap + X0);
 #pragma unroll 4
             for (int t = 0; t < trips; ++t) {
@@ -992,7 +1003,7 @@ __device__ __forceinline__ void block_planes_tc(const PassArgs &a, const TileGeo
                 ya += 2 * ap;
                 pb += bp;
             }
-        } else {
+        } else if (REST) {
             // other even sizes (and one tile of sy): k8 steps; columns past
             // the block (uneven G) enter as zeros
             const uint16_t *pa[NT];
@@ -1417,8 +1428,9 @@ __device__ __forceinline__ float stencil_reduce(const float (&acc)[5], int lane)
 // accumulators; dpart[(wi ng + gr) 5 + p] holds a group's partial sum.  TC: the
 // 16-bit path, where every window needs all five (16 pairs of 1 MP: 64 px 692 ->
 // 656 us, 32 px 487 -> 466, 16 px 549 -> 519 with the wider copies and fragment
-// loads); the FP32 kernels, where few do, keep the shorter code.
-template <bool TC>
+// loads); the FP32 kernels, where few do, keep the shorter code.  UNROLLED: the windows
+// (16, 32, 64 px, or-ed) that run the unrolled sums.
+template <bool TC, int UNROLLED>
 static __device__ __forceinline__ void stencil_direct(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs,
                                       const WinShared &ws)
 {
@@ -1439,11 +1451,11 @@ static __device__ __forceinline__ void stencil_direct(const PassArgs &a, const T
         // B' at A pixel (r, x) and shift (sy, sx): row r + sy + R + 1, column x + sx + padl
         const float *bbase = Bs + (wyi * g.s + r0 + ky + R + 1) * bpt + P.padl + wxi * g.s + kx;
         float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        if (TC && need == 0x1f && w == 16) {
+        if ((UNROLLED & 16) && need == 0x1f && w == 16) {
             stencil_sums<16>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
-        } else if (TC && need == 0x1f && w == 32) {
+        } else if ((UNROLLED & 32) && need == 0x1f && w == 32) {
             stencil_sums<32>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
-        } else if (TC && need == 0x1f && w == 64) {
+        } else if ((UNROLLED & 64) && need == 0x1f && w == 64) {
             stencil_sums<64>(abase, bbase, P.a_pitch, bpt, r1 - r0, lane, acc);
         } else if (need == 0x1f) {
             for (Walk2D e(lane, 32, w); e.y < r1 - r0; e.next()) {
@@ -1654,7 +1666,7 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
         else
             block_planes_fp32_generic(a, g, As, Bs, Ps);
     } else {
-        block_planes_tc<(RC >= 0 ? RC : 0), PREC>(a, g, TA, TB, Ps);
+        block_planes_tc<(RC >= 0 ? RC : 0), PREC, GC>(a, g, TA, TB, Ps);
     }
     __syncthreads();
     if (PREC != PREC_FP32 && P.RGx > 1) {
@@ -1666,16 +1678,17 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     constexpr bool tc = PREC != PREC_FP32;
     // two windows per warp once the tile has at least two per warp (16 px
     // tiles: 1.207 -> 1.198 ms per 64-pair launch; with fewer windows the
-    // warps left idle cost more than the shared set-up saves)
+    // warps left idle cost more than the shared set-up saves); on the 16-bit
+    // path up to r = 4 (registers)
     bool needs;
-    if (RC >= 0 && g.nwin >= 2 * (int)(blockDim.x >> 5))
+    if (RC >= 0 && (!tc || RC <= 4) && g.nwin >= 2 * (int)(blockDim.x >> 5))
         needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0), tc>(a, g, Ps, Vs, stats, ws, moff);
     else
         needs = plane_and_peak<RC, PREC == PREC_FP32 && (RC > SPREAD_MAX_R)>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
     // the direct stencil and its barrier only when some window needs them
     // (peaks at the edge of the search, and every window on the 16-bit path)
     if (__syncthreads_or(needs)) {
-        stencil_direct<tc>(a, g, As, Bs, ws);
+        stencil_direct<tc, tc && (GC != BLOCKS_ANY || !tc_split(RC)) ? 16 | 32 | 64 : 0>(a, g, As, Bs, ws);
         __syncthreads();
     }
     finalize(a, g, Vs, stats, ws, pair);
@@ -1767,7 +1780,7 @@ __global__ void __launch_bounds__(PASS_THREADS, GC == 32 ? 3 : 4) strip_kernel(c
         // 4: plane, argmax, FP32 stencil, Gaussian fit, outputs
         // the direct stencil and its barrier only when some window needs them
         if (__syncthreads_or(plane_and_peak<RC, true>(a, g, Ps, Vs, stats, false, ws, wy))) {
-            stencil_direct<false>(a, g, As, Bs, ws);
+            stencil_direct<false, 0>(a, g, As, Bs, ws);
             __syncthreads();
         }
         // the regions are read no more in this step: the next step's copies go

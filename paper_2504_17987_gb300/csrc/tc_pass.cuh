@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(PASS_THREADS, 2) tc_pass_kernel(const __grid_c
     // 5: argmax on the planes, FP32 five-point refit, Gaussian fit, outputs
     tc_plane_and_peak(a, g, Ps, Qs, Vs, stats, m, ws);
     __syncthreads();
-    stencil_direct<false>(a, g, As, Bs, ws);
+    stencil_direct<false, 0>(a, g, As, Bs, ws);
     __syncthreads();
     finalize(a, g, Vs, stats, ws, pair);
 }
