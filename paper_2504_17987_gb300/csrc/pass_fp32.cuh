@@ -86,13 +86,18 @@ static cudaError_t launch_radius_impl(const PassArgs &a, dim3 grid, int smem, cu
         default: break;
         }
     }
-    return launch_shape<RC, 0>(a, grid, smem, st);
+    // the unrolled loops of the usual blocks apart from the rest: in one kernel they spilled, and
+    // blocks of 4 px paid 3 to 7 % for them and their order of the units (16 px at 75 %, r = 4,
+    // 16 pairs of 1 MP: 1110 us apart, 1159 in one)
+    if (fp32_usual_blocks(G)) return launch_shape<RC, BLOCKS_USUAL>(a, grid, smem, st);
+    return launch_shape<RC, BLOCKS_ANY>(a, grid, smem, st);
 }
 
 template <int RC>
 static void prepare_radius_impl()
 {
-    prepare_shape<RC, 0>();
+    prepare_shape<RC, BLOCKS_ANY>();
+    prepare_shape<RC, BLOCKS_USUAL>();
     prepare_shape<RC, 8>();
     prepare_shape<RC, 12>();
     prepare_shape<RC, 16>();

@@ -646,6 +646,12 @@ __device__ __forceinline__ void sum_row_groups(float (&acc)[ND], int lrg)
     }
 }
 
+// Block sizes of a kernel that is not specialised to one (GC <= 0): any, or, at the radii
+// and types that have a kernel of their own for them, BLOCKS_USUAL (FP32: 8, 12, 16 and
+// 24 px) or BLOCKS_SLAB (16-bit, see tc_slab_blocks) in one and the rest in the other.
+constexpr int BLOCKS_ANY = 0, BLOCKS_USUAL = -1, BLOCKS_SLAB = -1;
+constexpr bool fp32_usual_blocks(int G) { return G == 8 || G == 12 || G == 16 || G == 24; }
+
 // Unit u of the plane loop as (block, shift row): whole groups of eight shift
 // rows of a block first, then every block's remaining ones.  The pitch of B' is
 // 4 x odd floats, so the 128-bit loads of a quarter-warp whose lanes take eight
@@ -695,7 +701,13 @@ __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileG
     // repeat it and store nothing
     for (int base = (threadIdx.x - lane) >> lrg; base < units; base += blockDim.x >> lrg) {
         int b, syi;
-        plane_unit<ND>(min(base + ul, units - 1), nblk, b, syi);
+        const int u = min(base + ul, units - 1);
+        if (GT > 0 || G >= 8) {
+            plane_unit<ND>(u, nblk, b, syi);
+        } else {
+            b = u / ND;
+            syi = u - b * ND;
+        }
         b += b0;
         const int byi = b / g.nbx, bxi = b - byi * g.nbx;
         const int c0 = bxi * G, r0 = byi * G + gi * rows;
@@ -783,18 +795,16 @@ __device__ __forceinline__ void block_planes_fp32(const PassArgs &a, const TileG
     }
 }
 
-// The plane loop of a kernel that is not specialised to one block size: the
-// block sizes of the usual windows (16 to 64 px at 50 % overlap, 32 to 96 px at
-// 75 %) run the unrolled loop.
+// The plane loop of the kernel for the block sizes of the usual windows (16 to 64 px
+// at 50 % overlap, 32 to 96 px at 75 %) in other shapes: unrolled.
 template <int R>
-__device__ __forceinline__ void block_planes_fp32_any(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs, float *Ps)
+__device__ __forceinline__ void block_planes_fp32_usual(const PassArgs &a, const TileGeom &g, const float *As, const float *Bs, float *Ps)
 {
     switch (g.G) {
     case 8: block_planes_fp32<R, 8>(a, g, As, Bs, Ps); return;
     case 12: block_planes_fp32<R, 12>(a, g, As, Bs, Ps); return;
     case 16: block_planes_fp32<R, 16>(a, g, As, Bs, Ps); return;
-    case 24: block_planes_fp32<R, 24>(a, g, As, Bs, Ps); return;
-    default: block_planes_fp32<R, 0>(a, g, As, Bs, Ps); return;
+    default: block_planes_fp32<R, 24>(a, g, As, Bs, Ps); return;
     }
 }
 
@@ -832,7 +842,7 @@ static __device__ __forceinline__ void block_planes_fp32_generic(const PassArgs 
         }
         sum_row_groups<8>(acc, lrg);
         if (base + ul < units && gi == 0) {
-            float *out = Ps + b * P.pstride + syi * ND + d0;
+            float *out = Ps + b * g.NP + syi * ND + d0;
             for (int d = 0; d < 8 && d0 + d < ND; ++d) out[d] = acc[d];
         }
     }
@@ -897,7 +907,6 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t &d0, uint32_t &d1, uint32_t
 // unrolled stencils or pairs of windows beyond r = 4.  As one kernel the code of the other
 // sizes spilled and cost the rest 1 to 3.5 % (16 pairs of 1 MP, r = 6: 24 px at 50 % 1122
 // us, 12 px 1990; as two 1086 and 1861; 32 px, of the slab blocks, 922 -> 759).
-constexpr int BLOCKS_ANY = 0, BLOCKS_SLAB = -1;
 constexpr bool tc_split(int R) { return R >= 4; }
 constexpr bool tc_slab_blocks(int R, int G) { return G % 16 == 0 || (G == 8 && (2 * R + 8) / 8 == 2); }
 
@@ -1170,8 +1179,8 @@ struct WinShared {
 // step passes the predictor through for them.
 // RC >= 0: compile-time radius; each lane decodes the shifts it owns
 // (q = lane + 32 j) once, into plane and box-sum offsets kept in registers.
-// ONE_PLANE: planes NP floats apart (strips, and tiles whose plan is never
-// spread); otherwise the plan's stride, which the planes were written at.
+// ONE_PLANE: planes NP floats apart (FP32 kernels whose plan is never spread); otherwise
+// the plan's stride.
 // ring_wy >= 0: strip mode, the window's block rows yy sit in ring rows
 // (ring_wy + yy) & 1.  Returns whether this thread stored a nonzero
 // direct-sum mask (some window needs the direct stencil).
@@ -1284,7 +1293,8 @@ static __device__ __forceinline__ bool plane_and_peak(const PassArgs &a, const T
 // key, then q): the largest value, ties to the smallest row-major index, NaN
 // never winning.  Results as plane_and_peak.
 // tc: 16-bit planes (moff, and every stencil point by the direct sums), as there.
-template <int RC, bool TC>
+// ONE_PLANE: as there.
+template <int RC, bool TC, bool ONE_PLANE>
 static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, const TileGeom &g, const float *Ps,
                                             const float *Vs, const float *stats, const WinShared &ws,
                                             float moff = 0.f)
@@ -1297,7 +1307,7 @@ static __device__ __forceinline__ bool plane_and_peak_pairs(const PassArgs &a, c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int h = lane >> 4, hl = lane & 15;
     const int kb = g.kb, sg = g.s / g.G;
-    const int ps = P.pstride, rs = g.nbx * ps;
+    const int ps = ONE_PLANE ? NP : P.pstride, rs = g.nbx * ps;
     const float tau = TAU_PER_PIXEL * (float)(g.w * g.w);
     const int cp = P.v_pitch;
     const float2 *VV = reinterpret_cast<const float2 *>(Vs);
@@ -1661,8 +1671,10 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     if (PREC == PREC_FP32) {
         if (RC >= 0 && GC > 0)
             block_planes_fp32<(RC >= 0 ? RC : 0), GC>(a, g, As, Bs, Ps);
+        else if (RC >= 0 && GC == BLOCKS_USUAL)
+            block_planes_fp32_usual<(RC >= 0 ? RC : 0)>(a, g, As, Bs, Ps);
         else if (RC >= 0)
-            block_planes_fp32_any<(RC >= 0 ? RC : 0)>(a, g, As, Bs, Ps);
+            block_planes_fp32<(RC >= 0 ? RC : 0), 0>(a, g, As, Bs, Ps);
         else
             block_planes_fp32_generic(a, g, As, Bs, Ps);
     } else {
@@ -1680,11 +1692,12 @@ __global__ void __launch_bounds__(PASS_THREADS, pass_ctas(RC, PREC, GC))
     // tiles: 1.207 -> 1.198 ms per 64-pair launch; with fewer windows the
     // warps left idle cost more than the shared set-up saves); on the 16-bit
     // path up to r = 4 (registers)
+    constexpr bool one_plane = !tc && !(GC > 0 && RC <= SPREAD_MAX_R);
     bool needs;
     if (RC >= 0 && (!tc || RC <= 4) && g.nwin >= 2 * (int)(blockDim.x >> 5))
-        needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0), tc>(a, g, Ps, Vs, stats, ws, moff);
+        needs = plane_and_peak_pairs<(RC >= 0 ? RC : 0), tc, one_plane>(a, g, Ps, Vs, stats, ws, moff);
     else
-        needs = plane_and_peak<RC, PREC == PREC_FP32 && (RC > SPREAD_MAX_R)>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
+        needs = plane_and_peak<RC, one_plane>(a, g, Ps, Vs, stats, tc, ws, -1, moff);
     // the direct stencil and its barrier only when some window needs them
     // (peaks at the edge of the search, and every window on the 16-bit path)
     if (__syncthreads_or(needs)) {

@@ -393,8 +393,8 @@ bool plan_search(int w, int s, int R, int G, int nx, int ny, int prec, PassPlan 
             }
         }
     if (pick_tx == 0) return false;
-    if (prec == PREC_FP32 && R <= SPREAD_MAX_R && fp32_radius_kernel(R, G) && pick_tx * pick_ty >= 2 * kThreads / 32) {
-        // tiles of the paired peak search (kernels with a compile-time radius): spread where it costs no CTA (16 px windows,
+    if (prec == PREC_FP32 && R <= SPREAD_MAX_R && fp32_shape_kernel(w, s, R, G) && pick_tx * pick_ty >= 2 * kThreads / 32) {
+        // tiles of the paired peak search in the kernels of one shape: spread where it costs no CTA (16 px windows,
         // r = 4, 64 pairs of 1 MP: 853 -> 824 us).  At r = 6 and 8 tiles seldom have 16
         // windows, and a stride known only at run time cost 0.5 %.
         const Layout L = layout_for(pick_tx, pick_ty, w, s, R, G, prec, false, true);

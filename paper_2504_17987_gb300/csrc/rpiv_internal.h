@@ -68,9 +68,16 @@ __device__ __forceinline__ const void *resolve(const PtrRef &r, int pair)
 // the kernel of any radius serves the rest.  Read by the dispatch and by the planner.
 constexpr bool fp32_radius_kernel(int R, int G) { return G % 4 == 0 && ((R >= 0 && R <= 4) || R == 6 || R == 8); }
 
+// Block sizes of the FP32 kernels specialised to 50 % overlap (radii 1 to 8 of the above).
+constexpr bool fp32_shape_kernel(int w, int s, int R, int G)
+{
+    return fp32_radius_kernel(R, G) && R > 0 && w == 2 * G && s == G &&
+           (G == 8 || G == 12 || G == 16 || G == 24 || G == 32);
+}
+
 // Largest radius whose FP32 tiles may have their planes spread (PassPlan::pstride
-// above the plane's size); the kernels of larger compile-time radii hold the
-// stride as a constant.
+// above the plane's size), and only for the kernels specialised to their shape;
+// every other kernel holds the stride as the plane's size.
 constexpr int SPREAD_MAX_R = 4;
 
 struct PassPlan {
