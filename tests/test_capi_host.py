@@ -66,3 +66,8 @@ def test_only_later_parts_uploads_make_room_for_passes(probe):
     # the first part's upload runs before any pass, with the device to itself
     res = probe("".join(f"batch {FRAMES[1]} {n} 1 -1\n" for n in (1, 2, 4, 33)))
     assert [r[3] for r in res] == [r[1] - 1 for r in res] == [0, 1, 3, 3]
+
+
+def test_parts_too_small_to_be_cut_upload_side_by_side(probe):
+    # 17 frames of 0.2 MB: two parts, neither of which waits for the other's upload or makes room for it
+    assert probe("batch 519 403 17 1 -1\n") == [[0, 2, 0, 0]]
