@@ -894,6 +894,23 @@ static std::vector<BatchPart> batch_parts(int n, size_t upload_bytes_per_pair)
 static bool parts_conflict(const PairIO *io, const std::vector<BatchPart> &parts, size_t count)
 {
     auto at = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+    // the usual call first: no predictor within the span of the fields or of the masks
+    const int n = parts.back().first + parts.back().count;
+    uintptr_t lo[2] = {UINTPTR_MAX, UINTPTR_MAX}, hi[2] = {0, 0};
+    auto span = [&](const void *p, size_t bytes, int k) {
+        if (!p) return;
+        lo[k] = std::min(lo[k], at(p));
+        hi[k] = std::max(hi[k], at(p) + bytes);
+    };
+    for (const PairIO *p = io; p < io + n; ++p) {
+        for (const float *f : {p->u, p->v, p->vort}) span(f, 4 * count, 0);
+        span(p->mask, count, 1);
+    }
+    bool near = false;
+    for (const PairIO *p = io; p < io + n; ++p)
+        for (const float *f : {p->pred_u, p->pred_v})
+            for (int k = 0; f && k < 2; ++k) near |= at(f) < hi[k] && at(f) + 4 * count > lo[k];
+    if (!near) return false;
     std::vector<std::pair<uintptr_t, uintptr_t>> out;
     for (const BatchPart &w : parts) {
         out.clear();
