@@ -1043,8 +1043,11 @@ def main():
 def kernel_bytes(rec: dict, bpp: int, margin: int) -> int | None:
     """Algorithmic DRAM bytes of one traced launch (the data the step must
     move, independent of how the kernel schedules it): frames read once and
-    written once, node fields read and written once.  rec: a stage-trace record
-    (name, pairs, image size, grid)."""
+    written once, node fields read and written once.  A deformation's predictor
+    fields (16 bytes a node, at most 4 % of its frames) are left out.  rec: a
+    stage-trace record (name, pairs, image size, grid); the library traces
+    frames/*, deform/*, pass/*, uod/* and vort, and upload with host frames; the
+    other names are those of stages that it once launched by themselves."""
     name, n, W, H = rec["name"], rec["pairs"], rec["width"], rec["height"]
     nodes = rec["nx"] * rec["ny"]
     if name == "ingest":  # u8/u16 frame in, float frame (interior) out

@@ -19,7 +19,8 @@
 //      bilinear weights, along x and then y                         -> grad
 // One 1 MP pair moves a few megabytes through L2: the chain is bound by the
 // latency of its launches, so there are three (two for the score alone).  As
-// seven launches it took 73 us (125 x 125 nodes, score and gradient); now 29.
+// seven launches it took 73 us (125 x 125 nodes, score and gradient); now 30, of which
+// the host's side of the call is 25.
 // Blocks above 32 px, steps below 3 px and steps whose node tiles do not fit shared memory run
 // steps 1 and 3 as separate launches over pixels, rows and nodes.
 #include <algorithm>

@@ -98,7 +98,8 @@ __device__ __forceinline__ const T *tap(const T *base, long long pe, int x, int 
 //   - when every lane's four rows have the same integer displacement (a smooth
 //     field between its integer steps), their taps are five consecutive source
 //     rows: ten loads instead of sixteen.
-// 64 pairs of 1 MP, 16 px windows: 193 -> 170 us (0.32 -> 0.36 of the HBM rate).
+// 64 pairs of 1 MP, 16 px windows: 193 -> 170 us (0.32 -> 0.36 of the HBM rate); 181
+// (0.34) since the launch also interpolates its predictor.
 // CLAMP: the taps are clamped to the image (tiles near its border or with a
 // displacement range reaching outside); otherwise the taps are read from one
 // base pointer.  Off: the integer type of pixel offsets.
@@ -391,9 +392,10 @@ static void launch_tiles(const DeformArgs &a, int n_pairs, cudaStream_t st)
     else launch_tiles_caps<DTY, 3>(a, n_pairs, st);
 }
 
-// 64 x 128 tiles when they still make two full waves (five CTAs per SM on
-// 152 SMs): 0.235 -> 0.215 ms per 64-pair 1 MP launch; smaller launches take
-// the tallest tile that still gives four CTAs per SM, at least 64 x 32
+// 64 x 128 tiles when there are ten of them per SM, a wave and two thirds at the
+// kernel's six CTAs per SM (the line was drawn at two waves of five: 0.235 ->
+// 0.215 ms per 64-pair 1 MP launch); smaller launches take the tallest tile that
+// still gives four CTAs per SM, at least 64 x 32
 cudaError_t launch_deform(const DeformArgs &a, int n_pairs, cudaStream_t st)
 {
     const long long WE = a.W + 2LL * a.M, HE = a.H + 2LL * a.M;
