@@ -1,9 +1,9 @@
 """The distance between a tile's block planes, on the host: pass_plan.cpp built with
 the host compiler against stub launchers.  Only tiles of the paired peak search in a
-kernel with a compile-time radius (blocks a multiple of 4 px, radii 0 to 4) may have
-their planes spread; everywhere else consecutive planes are their own size apart (a
-16-bit tile's row groups keep their partial planes beside one another)."""
-import math
+kernel specialised to its shape (50 % overlap, blocks of 8, 12, 16, 24 or 32 px, radii 1
+to 4) may have their planes spread: the other kernels hold the distance as a constant,
+the planes' own size (a 16-bit tile's row groups keep their partial planes beside one
+another)."""
 import os
 import shutil
 import subprocess
@@ -48,7 +48,7 @@ def test_planes_are_spread_only_for_kernels_that_read_them_so(tmp_path):
         if not ok:
             continue
         size = (2 * R + 1) ** 2
-        if prec == 0 and math.gcd(w, s) % 4 == 0 and R <= 4 and TX * TY >= 2 * THREADS // 32:
+        if prec == 0 and w == 2 * s and s in (8, 12, 16, 24, 32) and 1 <= R <= 4 and TX * TY >= 2 * THREADS // 32:
             assert pstride >= size
             spread += pstride > size
         else:
