@@ -342,6 +342,15 @@ __global__ void __launch_bounds__(256) adj_blocks(const AdjArgs a, const AdjWs w
     __syncthreads();
     const int l = tid & (lanes - 1), nb = nbx * nby;
     const float inv_n = 1.f / (float)(G * G);
+    // means are summed relative to the least of the tile's corners, so that a background's
+    // offset does not take the sums' digits (sparse particles on 100 counts, 32 px at 75 %:
+    // gradient error 0.9e-6 instead of 1.35e-6)
+    auto base = [&](const float *v) {
+        const float *w = v + (ph - 1) * pitch;
+        const float m = fminf(fminf(v[0], v[pw - 1]), fminf(w[0], w[pw - 1]));
+        return isfinite(m) ? m : 0.f;
+    };
+    const float ra = base(sa), rb = base(sb);
     // warp-uniform trip count for the shuffles; threads past the last block repeat it
     for (int k0 = 0; k0 < nb; k0 += blockDim.x / lanes) {
         const int k = k0 + tid / lanes, kc = min(k, nb - 1);
@@ -351,15 +360,15 @@ __global__ void __launch_bounds__(256) adj_blocks(const AdjArgs a, const AdjWs w
         for (int x = l, y = 0;; x += lanes) {
             for (; x >= G; x -= G) ++y;
             if (y >= G) break;
-            m0 += pa[y * pitch + x];
-            m1 += pb[y * pitch + x];
+            m0 += pa[y * pitch + x] - ra;
+            m1 += pb[y * pitch + x] - rb;
         }
         for (int o = lanes >> 1; o > 0; o >>= 1) {
             m0 += __shfl_xor_sync(0xffffffffu, m0, o);
             m1 += __shfl_xor_sync(0xffffffffu, m1, o);
         }
-        m0 *= inv_n;
-        m1 *= inv_n;
+        m0 = fmaf(m0, inv_n, ra);
+        m1 = fmaf(m1, inv_n, rb);
         float caa = 0.f, cbb = 0.f, cab = 0.f;
         for (int x = l, y = 0;; x += lanes) {
             for (; x >= G; x -= G) ++y;
@@ -421,16 +430,17 @@ __global__ void __launch_bounds__(256) adj_block_kernel(const AdjArgs a, const A
     const int G = bg.G, n = G * G;
     const float4 *p = ws.px4 + (long long)(by * G) * a.W + bx * G;
     const int start = own * 32 + lane;
+    const float4 f = *p;  // the means are summed relative to the first pixel (offsets)
     float sa = 0.f, sb = 0.f;
     for (Walk e(start, 32 * WARPS, G); e.y < G; e.next()) {
         const float4 v = p[(long long)e.y * a.W + e.x];
-        sa += v.w;
-        sb += v.x;
+        sa += v.w - f.w;
+        sb += v.x - f.x;
     }
     sa = put(sa, 0);
     sb = put(sb, 1);
     if (WARPS > 1) __syncthreads();
-    const float ma = get(sa, 0) / (float)n, mb = get(sb, 1) / (float)n;
+    const float ma = f.w + get(sa, 0) / (float)n, mb = f.x + get(sb, 1) / (float)n;
     float caa = 0.f, cbb = 0.f, cab = 0.f;
     for (Walk e(start, 32 * WARPS, G); e.y < G; e.next()) {
         const float4 v = p[(long long)e.y * a.W + e.x];
