@@ -472,15 +472,21 @@ __device__ __forceinline__ void score_sum(const AdjArgs &a, const AdjWs &ws, int
 
 // 2: per window, its (w/G)^2 blocks combined: equal-size parts, so the mean
 // is the mean of the block means, and each centred moment gains
-// G^2 sum (mean_k - mean)(mean'_k - mean').  Two passes: the mean, then
+// G^2 sum (mean_k - mean)(mean'_k - mean').  Two passes: a reference near the mean
+// (the mean up to 4 x 4 blocks, that of four whole block rows above), then
 // sum (d - mean d)^2 = sum d^2 - (sum d)^2 / k with d relative to it, whose second term
-// only mends the mean's rounding.  (With d relative to the window's first block in one
-// pass the two terms cancelled: score error against 64 bits 3.0e-7 instead of 2e-8 with
-// 64 px windows at 6 px steps, gradient error 3.0e-6 instead of 2.2e-6 with 16 px windows
-// at 5 px steps on sparse particles; relative to a mean of sixteen blocks 5.0e-7, whose few
-// bits make the dark pixels' equal terms round all to one side.)
+// is small.  (With d relative to the window's first block the two terms cancelled:
+// score error against 64 bits 3.0e-7 instead of 2e-8 with 64 px windows at 6 px steps,
+// gradient error 3.0e-6 instead of 2.2e-6 with 16 px windows at 5 px steps on sparse
+// particles; relative to a mean of sixteen blocks 5.0e-7, whose few bits make the dark
+// pixels' equal terms round all to one side.)
 // The block rows of a window are dealt to WIN_LANES lanes and added by shuffles,
 // so that its loads are in flight together.
+// FEW: windows of up to 4 x 4 blocks (50 and 75 % overlap among them): a lane's row stays
+// in registers, one latency for both passes.  A kernel of its own: the loops of larger
+// windows want the CTAs that its registers cost (score of a 1 MP pair, 64 px at 4 px
+// steps: 90 us in one, 71 apart, and 60 with the reference from four rows).
+template <bool FEW>
 __global__ void __launch_bounds__(WIN_CTA *WIN_LANES) adj_windows(const AdjArgs a, const AdjWs ws, const BlockGrid bg,
                                                                     bool sum_here)
 {
@@ -500,7 +506,7 @@ __global__ void __launch_bounds__(WIN_CTA *WIN_LANES) adj_windows(const AdjArgs 
         };
         static_assert(WIN_LANES == 4, "two shuffles, a row each up to 4 x 4 blocks");
         const float inv_k = 1.f / (float)(kb * kb), nb = (float)(G * G);
-        // the blocks' mean, then the moments relative to it
+        // the reference, then the moments relative to it
         float2 f = make_float2(0.f, 0.f);
         float da = 0.f, db = 0.f, daa = 0.f, dbb = 0.f, dab = 0.f, ea = 0.f, eb = 0.f, num = 0.f;
         auto moments = [&](const float4 &o, float ab) {
@@ -514,7 +520,7 @@ __global__ void __launch_bounds__(WIN_CTA *WIN_LANES) adj_windows(const AdjArgs 
             eb += o.w;
             num += ab;
         };
-        if (kb <= 4) {  // 50 and 75 % overlap among them: a lane's row stays in registers, one latency for both passes
+        if (FEW) {
             float4 o[4];
             float ab[4];
 #pragma unroll
@@ -532,15 +538,15 @@ __global__ void __launch_bounds__(WIN_CTA *WIN_LANES) adj_windows(const AdjArgs 
             for (int p = 0; p < 4; ++p)
                 if (l < kb && p < kb) moments(o[p], ab[p]);
         } else {
-            for (int q = l; q < kb; q += WIN_LANES)
+            const int q0 = (l * kb) >> 2;
 #pragma unroll 4
-                for (int p = 0; p < kb; ++p) {
-                    const float2 o = *reinterpret_cast<const float2 *>(ws.blk + b0 + q * bg.nbx + p);
-                    f.x += o.x;
-                    f.y += o.y;
-                }
-            f.x = all(f.x) * inv_k;
-            f.y = all(f.y) * inv_k;
+            for (int p = 0; p < kb; ++p) {
+                const float2 o = *reinterpret_cast<const float2 *>(ws.blk + b0 + q0 * bg.nbx + p);
+                f.x += o.x;
+                f.y += o.y;
+            }
+            f.x = all(f.x) * (1.f / (float)(4 * kb));
+            f.y = all(f.y) * (1.f / (float)(4 * kb));
             for (int q = l; q < kb; q += WIN_LANES)
 #pragma unroll 4
                 for (int p = 0; p < kb; ++p) {
@@ -841,7 +847,8 @@ cudaError_t run(const AdjArgs &a, cudaStream_t st)
     const NodeTile t = node_tile(a.W, a.H, a.w, a.s, a.nx, a.ny);
     const int wc = win_ctas(a.nx, a.ny);
     const bool sum_in_nodes = grad && t.ok;
-    adj_windows<<<wc, WIN_CTA * WIN_LANES, 0, st>>>(a, ws, bg, !sum_in_nodes);
+    if (a.w / bg.G <= 4) adj_windows<true><<<wc, WIN_CTA * WIN_LANES, 0, st>>>(a, ws, bg, !sum_in_nodes);
+    else adj_windows<false><<<wc, WIN_CTA * WIN_LANES, 0, st>>>(a, ws, bg, !sum_in_nodes);
     if (grad) {
         if (t.ok) {
             adj_nodes<<<dim3((a.nx + t.tx - 1) / t.tx, (a.ny + t.ty - 1) / t.ty), 256, t.smem, st>>>(a, ws, bg, t, a.score_out ? wc : 0);
